@@ -364,22 +364,32 @@ cudaError_t launch_qsig(int K, const CUtensorMap& mq, const CUtensorMap& mp, con
   return cudaErrorInvalidValue;
 }
 
-// `count_max` bounds every count (0 = no bound known): it lets the count stage skip radix passes
-// over bytes that are zero everywhere.
-laser_kv_status_t launch_select(SelectArgs a, int n_seg, uint32_t count_max, cudaStream_t st) {
-  static std::atomic<unsigned long long> limit_set{0};
-  const size_t smem = (size_t)a.S * 9;
-  if (ensure_smem_limit(limit_set, select_kernel, kMaxSmem - 2048) != cudaSuccess)
-    return fail(nullptr, LASER_KV_ERR_CUDA, "cudaFuncSetAttribute(select_kernel) failed");
-  int top_shift = 24;
-  if (count_max != 0) {
-    top_shift = 0;
-    while (top_shift < 24 && (count_max >> (top_shift + 8)) != 0) top_shift += 8;
-  }
-  a.count_top_shift = top_shift;
-  select_kernel<<<n_seg, kSelThreads, smem, st>>>(a);
+template <int T, int NI>
+cudaError_t launch_select_t(const SelectArgs& a, int n_seg, cudaStream_t st) {
+  static std::atomic<unsigned long long> limit_set{0};   // per instantiation
+  const cudaError_t e = ensure_smem_limit(limit_set, select_kernel<T, NI>, NI * T * 4);
+  if (e != cudaSuccess) return e;
+  select_kernel<T, NI><<<n_seg, T, (size_t)a.S * 4, st>>>(a);
   g_launches.fetch_add(1);
-  const cudaError_t e = cudaGetLastError();
+  return cudaGetLastError();
+}
+
+// A CTA of 1024 threads per segment: its barriers and its chains of shared-memory round trips set the
+// time, so the fewer keys a thread has the better. Segments of at most 4096 keys that outnumber the
+// SMs go to CTAs of 512 threads, two of which share an SM and hide each other's barriers (512 segments
+// of 4096 keys: 28.9 us; the row counts of the instances are spaced so that at most a third of the rows is empty).
+laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, cudaStream_t st) {
+  cudaError_t e;
+  if (a.S <= 4096 && n_seg > num_sms) {
+    e = a.S <= 1024 ? launch_select_t<512, 2>(a, n_seg, st) : a.S <= 2048 ? launch_select_t<512, 4>(a, n_seg, st)
+                                                                          : launch_select_t<512, 8>(a, n_seg, st);
+  } else {
+    const int ni = (a.S + 1023) / 1024;
+    e = ni <= 1 ? launch_select_t<1024, 1>(a, n_seg, st) : ni <= 2 ? launch_select_t<1024, 2>(a, n_seg, st)
+      : ni <= 4 ? launch_select_t<1024, 4>(a, n_seg, st) : ni <= 6 ? launch_select_t<1024, 6>(a, n_seg, st)
+      : ni <= 8 ? launch_select_t<1024, 8>(a, n_seg, st) : ni <= 10 ? launch_select_t<1024, 10>(a, n_seg, st)
+      : ni <= 16 ? launch_select_t<1024, 16>(a, n_seg, st) : launch_select_t<1024, 24>(a, n_seg, st);
+  }
   if (e != cudaSuccess) return fail(nullptr, LASER_KV_ERR_CUDA, "select_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }
@@ -553,7 +563,7 @@ namespace {
 struct CallGeom {
   int S_len;                 // scored keys per segment
   int shift;                 // rows before the block's first token that belong to the segment (0 or anchors)
-  int keep_a_lo, keep_a_hi, keep_b_lo, keep_b_hi, excl_lo, excl_hi, cand_lo, cand_hi;   // scored-key index ranges
+  int keep_a_lo, keep_a_hi, keep_b_lo, keep_b_hi, excl_lo, excl_hi;   // scored-key index ranges
   int k_exact, k_lsh;
   int B_out;                 // cache entries per block and head
   int S_tok;                 // tokens per block of this pass (the block size; fewer for a short last block)
@@ -582,13 +592,11 @@ CallGeom make_geom(int S_tok, int B, int n, double alpha, bool lookback, int rel
     g.S_len = S_tok; g.shift = 0;
     g.keep_a_lo = 0; g.keep_a_hi = a; g.keep_b_lo = S_tok - a; g.keep_b_hi = S_tok;
     g.excl_lo = g.excl_hi = 0;
-    g.cand_lo = a; g.cand_hi = S_tok - a;
     g.B_out = B;
   } else {
     g.S_len = S_tok + released; g.shift = released;
     g.keep_a_lo = released; g.keep_a_hi = released + a; g.keep_b_lo = g.keep_b_hi = 0;
     g.excl_lo = released + S_tok - a; g.excl_hi = released + S_tok;
-    g.cand_lo = 0; g.cand_hi = released + S_tok - a;
     g.B_out = a + b_long;
   }
   return g;
@@ -772,10 +780,10 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
   //    settles its own list first), then the two-stage top-k
   {
     SelectArgs sel{s_exact, counts, idx, S_len, g.k_exact, g.k_lsh, g.keep_a_lo, g.keep_a_hi, g.keep_b_lo, g.keep_b_hi,
-                   g.excl_lo, g.excl_hi, g.cand_lo, g.cand_hi, 0, need_lsh ? 1 : 0,
+                   g.excl_lo, g.excl_hi, need_lsh ? 1 : 0,
                    SignfixArgs{K0, kv_strides[0], kv_strides[1], kv_strides[2], h->P, hist, counts, key_buckets, fix_items,
                                fix_counts, d.fix_cap, c.n_kv_heads, nb, S_len, d.Kp, d.Lp, ctrl + 2, S, ctrl + 1}};
-    const laser_kv_status_t s = launch_select(sel, nseg, (uint32_t)d.GW * (uint32_t)d.Lp, st);
+    const laser_kv_status_t s = launch_select(sel, nseg, h->num_sms, st);
     if (s != LASER_KV_OK) { h->last_error = g_last_error; return s; }
   }
   mark();
@@ -1323,8 +1331,13 @@ laser_kv_status_t laser_kv_two_stage_topk(const float* s_exact, const uint32_t* 
     return fail(nullptr, LASER_KV_ERR_INVALID_ARG, "two_stage_topk: keep count exceeds the segment");
   if (S > 16384) return fail(nullptr, LASER_KV_ERR_UNSUPPORTED, "two_stage_topk: S > 16384");
   if (2 * anchors + k_exact + k_lsh == 0) return LASER_KV_OK;
-  const SelectArgs sel{s_exact, counts, idx_out, S, k_exact, k_lsh, 0, anchors, S - anchors, S, 0, 0, anchors, S - anchors, 0};
-  return launch_select(sel, n_segments, 0u, static_cast<cudaStream_t>(stream));
+  const SelectArgs sel{s_exact, counts, idx_out, S, k_exact, k_lsh, 0, anchors, S - anchors, S, 0, 0, 0};
+  int dev = 0, num_sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return fail(nullptr, LASER_KV_ERR_CUDA, "two_stage_topk: device query: %s", cudaGetErrorString(e));
+  return launch_select(sel, n_segments, num_sms, static_cast<cudaStream_t>(stream));
 }
 
 // ---- window scores on caller-fed inputs ----------------------------------------------------------

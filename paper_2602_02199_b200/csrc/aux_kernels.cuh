@@ -1,8 +1,8 @@
 // The non-GEMM kernels of the selection path:
 //   signfix_kernel - exact recomputation of key sign bits whose tensor-core projection was too
 //                    close to zero to trust, with the matching correction of the counts.
-//   select_kernel  - Algorithm 1 lines 4-8: two-stage top-k per (sequence, KV head, block) by
-//                    shared-memory radix selection, ties to the lower index, ascending output.
+//   select_kernel  - Algorithm 1 lines 4-8: two-stage top-k per (sequence, KV head, block) by radix
+//                    selection on registers, ties to the lower index, ascending output.
 //   append_kernel  - gather of the kept K/V rows into the append-only cache (16-byte vectors).
 #pragma once
 #include <cuda_runtime.h>
@@ -97,115 +97,163 @@ __global__ void __launch_bounds__(256) signfix_kernel(const SignfixArgs a) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Two-stage top-k. One CTA of 1024 threads per segment; scores and counts live in shared memory.
+// Two-stage top-k. One CTA of T threads per segment; thread t owns the keys t, t + T, t + 2T, ... and
+// holds their values of the running stage in registers, its candidate / kept flags as bit masks.
+//
+// Bound by barriers and by histogram atomics in shared memory, not by bytes (64 KB per segment of
+// 8192 keys). A radix round bins the values that are still undecided by the eleven highest bits in
+// which they can differ: the first round subtracts the smallest candidate, so that scores that share
+// their exponent bits do not pile up in a few bins (atomics of a warp on one bin go one by one), and
+// the k-th largest of 8192 scores is usually alone in its bin after two rounds, a count after one.
+// A round takes three barriers. Against 8-bit rounds over values and flags in shared memory (whole
+// kernel, doubtful signs included): 512 segments of 4096 keys 62 -> 29 us, 128 of 8192 25.2 -> 20.3 us,
+// 8 of 8192 22.2 -> 16.5 us, 80 of 1864 without signs 7.5 -> 4.7 us.
 // ------------------------------------------------------------------------------------------------
-constexpr int kSelThreads = 1024;
+constexpr int kSelBins = 2048;
+constexpr int kSelBinBits = 11;
+constexpr int kSelMaxKeys = 24 * 1024;   // a block of 16384 keys and the 8192 that look-back may hold back
 
 __device__ __forceinline__ uint32_t orderable_f32(float f) {
   const uint32_t u = __float_as_uint(f);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Exclusive scan of one int per thread over the whole CTA; `total` receives the sum.
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total) {
+template <int T, int NI>
+struct SelShared {
+  static constexpr int kWarps = T / 32;
+  int hist[kSelBins];              // all zero between rounds
+  int chunk_sum[kWarps];
+  int found[3];                    // bin, elements still needed from it, elements in it
+  uint32_t range[4][kWarps];       // per warp: smallest and largest score, smallest and largest count
+  int before[2][kWarps * NI];      // ordered_ranks: tie break, compaction
+};
+
+// For every row i of the CTA (keys i*T .. i*T + T - 1): how many keys of smaller index than the
+// calling warp's part of the row have their bit set in `mask` (bit i of a thread's mask: its key of
+// row i). Lane i of the warp receives the number for row i. Two barriers.
+template <int T, int NI>
+__device__ __forceinline__ int ordered_ranks(uint32_t mask, int* before) {
+  constexpr int NW = T / 32, E = NW * NI, PER = (E + 31) / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = v;
+  int mine = 0;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int n = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += n;
+  for (int i = 0; i < NI; ++i) {
+    const int n = __popc(__ballot_sync(0xffffffffu, (mask >> i) & 1u));
+    if (lane == i) mine = n;
   }
-  if (lane == 31) warp_sums[warp] = incl;
+  if (lane < NI) before[lane * NW + warp] = mine;
   __syncthreads();
   if (warp == 0) {
-    int s = warp_sums[lane];
-    int si = s;
+    int v[PER], sum = 0;
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      v[p] = (lane * PER + p < E) ? before[lane * PER + p] : 0;
+      sum += v[p];
+    }
+    int incl = sum;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const int n = __shfl_up_sync(0xffffffffu, si, off);
-      if (lane >= off) si += n;
+      const int n = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += n;
     }
-    warp_sums[lane] = si - s;          // exclusive warp offsets
-    if (lane == 31) warp_sums[32] = si;
+    int run = incl - sum;
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      if (lane * PER + p < E) before[lane * PER + p] = run;
+      run += v[p];
+    }
   }
   __syncthreads();
-  const int res = warp_sums[warp] + incl - v;
-  total = warp_sums[32];
-  __syncthreads();
-  return res;
+  return lane < NI ? before[lane * NW + warp] : 0;
 }
 
-// Among the participating elements j in [lo, hi) (flag[j] == 0) finds the k-th largest value T
-// (k >= 1, k <= number of participants) and how many elements equal to T belong to the top k.
-// `top_shift` is the position of the highest byte that can differ between values (24 for arbitrary
-// 32-bit keys); the bytes above it must be zero in every value.
-__device__ void radix_select_kth(const uint32_t* vals, const uint8_t* flag, int lo, int hi, int k, int top_shift,
-                                 int* hist, int* misc, uint32_t& T, int& need) {
-  uint32_t prefix = 0, mask = ~((top_shift >= 24) ? 0xFFFFFFFFu : ((1u << (top_shift + 8)) - 1u));
-  int remaining = k;
-  for (int shift = top_shift; shift >= 0; shift -= 8) {
-    for (int i = threadIdx.x; i < 256; i += kSelThreads) hist[i] = 0;
+// Moves the k largest values among the candidates (bit i of `cand`: v[i] takes part) from `cand` to
+// `kept`; equal values: lower index first. lo and hi bound the candidates' values; there are at
+// least k candidates.
+template <int T, int NI>
+__device__ __forceinline__ void take_topk(const uint32_t (&v)[NI], uint32_t& cand, uint32_t& kept, int k, uint32_t lo,
+                                          uint32_t hi, SelShared<T, NI>& sh) {
+  if (k <= 0) return;                    // uniform across the CTA
+  constexpr int NW = T / 32;
+  constexpr int PER = kSelBins / T;      // bins a thread sums up
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t in = cand, base = lo;         // still undecided; the smallest value they can have
+  int need = k, shift = 32 - __clz(hi - lo) - kSelBinBits;
+  if (shift < 0) shift = 0;
+  for (;;) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+      if ((in >> i) & 1u) atomicAdd(&sh.hist[(v[i] - base) >> shift], 1);
     __syncthreads();
-    for (int j = lo + threadIdx.x; j < hi; j += kSelThreads) {
-      if (!flag[j]) {
-        const uint32_t u = vals[j];
-        if ((u & mask) == prefix) atomicAdd(&hist[(u >> shift) & 255], 1);
-      }
+    // warp w sums the w-th highest run of 32 * PER bins; the lanes go from high bins to low ones
+    const int b0 = kSelBins - (warp * 32 + lane + 1) * PER;
+    int c[PER], sum = 0;
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      c[p] = sh.hist[b0 + PER - 1 - p];
+      sh.hist[b0 + PER - 1 - p] = 0;
+      sum += c[p];
     }
+    const int wsum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) sh.chunk_sum[warp] = wsum;
     __syncthreads();
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      int c[8], tot = 0;
+    {
+      const int x = lane < NW ? sh.chunk_sum[lane] : 0;
+      int incl = x;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) { c[i] = hist[255 - 8 * lane - i]; tot += c[i]; }
-      int incl = tot;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
+      for (int off = 1; off < NW; off <<= 1) {
         const int n = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += n;
       }
-      const int excl = incl - tot;       // elements with a larger digit than this lane's range
-      if (excl < remaining && remaining <= incl) {
-        int run = excl;
+      const int owner = __ffs(__ballot_sync(0xffffffffu, need <= incl)) - 1;
+      if (warp == owner) {               // this warp's bins hold the k-th value
+        int run = __shfl_sync(0xffffffffu, incl - x, owner);
+        int in_warp = sum;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (run < remaining && remaining <= run + c[i]) { misc[0] = 255 - 8 * lane - i; misc[1] = remaining - run; }
-          run += c[i];
+        for (int off = 1; off < 32; off <<= 1) {
+          const int n = __shfl_up_sync(0xffffffffu, in_warp, off);
+          if (lane >= off) in_warp += n;
+        }
+        run += in_warp - sum;            // elements in higher bins than this lane's
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+          if (run < need && need <= run + c[p]) {
+            sh.found[0] = b0 + PER - 1 - p;
+            sh.found[1] = need - run;
+            sh.found[2] = c[p];
+          }
+          run += c[p];
         }
       }
     }
     __syncthreads();
-    prefix |= (uint32_t)misc[0] << shift;
-    mask |= 0xFFu << shift;
-    remaining = misc[1];
-    __syncthreads();
+    const uint32_t bin = (uint32_t)sh.found[0];
+    need = sh.found[1];
+    const int held = sh.found[2];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const uint32_t d = (v[i] - base) >> shift, bit = in & (1u << i);
+      if (d != bin) in &= ~bit;
+      if (d > bin) kept |= bit;
+    }
+    if (need == held) {                  // the whole bin
+      kept |= in;
+      break;
+    }
+    if (shift == 0) {                    // equal values: the ones of lowest index
+      const int rank0 = ordered_ranks<T, NI>(in, sh.before[0]);
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const uint32_t row = __ballot_sync(0xffffffffu, (in >> i) & 1u);
+        const int rank = __shfl_sync(0xffffffffu, rank0, i) + __popc(row & ((1u << lane) - 1u));
+        if (rank < need) kept |= in & (1u << i);
+      }
+      break;
+    }
+    base += bin << shift;
+    shift = shift > kSelBinBits ? shift - kSelBinBits : 0;
   }
-  T = prefix;
-  need = remaining;
-}
-
-// Marks (flag = 1) the k largest participating elements of [lo, hi); equal values: lower index.
-__device__ void mark_topk(const uint32_t* vals, uint8_t* flag, int lo, int hi, int k, int top_shift, int* hist,
-                          int* misc, int* warp_sums) {
-  if (k <= 0) return;                    // uniform across the CTA
-  uint32_t T;
-  int need;
-  radix_select_kth(vals, flag, lo, hi, k, top_shift, hist, misc, T, need);
-  const int n = hi - lo;
-  const int per = (n + kSelThreads - 1) / kSelThreads;
-  const int j0 = lo + threadIdx.x * per;
-  const int j1 = min(hi, j0 + per);
-  int eq = 0;
-  for (int j = j0; j < j1; ++j) eq += (!flag[j] && vals[j] == T) ? 1 : 0;
-  int total;
-  int rank = block_exclusive_scan(eq, warp_sums, total);
-  for (int j = j0; j < j1; ++j) {
-    if (flag[j]) continue;
-    const uint32_t u = vals[j];
-    if (u > T) flag[j] = 1;
-    else if (u == T) { if (rank < need) flag[j] = 1; ++rank; }
-  }
-  __syncthreads();
+  cand &= ~kept;
 }
 
 // The S scored keys of a segment fall into three classes: kept whatever their scores (two index
@@ -218,46 +266,85 @@ struct SelectArgs {
   int S, k_exact, k_lsh;
   int keep_a_lo, keep_a_hi, keep_b_lo, keep_b_hi;   // kept ranges [lo, hi); empty when lo >= hi
   int excl_lo, excl_hi;                             // excluded range
-  int cand_lo, cand_hi;                             // a range that contains every candidate
-  int count_top_shift;      // highest byte position (0, 8, 16 or 24) in which two counts can differ
   int has_fix;              // nonzero: `fix` names the segment lists of doubtful key signs to settle first
   SignfixArgs fix;
 };
 
-__global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const SelectArgs a) {
+template <int T, int NI>
+__global__ void __launch_bounds__(T, 1024 / T) select_kernel(const SelectArgs a) {
   extern __shared__ uint8_t smem_sel[];
-  uint32_t* ukey = reinterpret_cast<uint32_t*>(smem_sel);
-  uint32_t* ucnt = ukey + a.S;
-  uint8_t* flag = reinterpret_cast<uint8_t*>(ucnt + a.S);
-  __shared__ int hist[256];
-  __shared__ int misc[2];
-  __shared__ int warp_sums[33];
-  const int seg = blockIdx.x;
-  const int S = a.S, lo = a.cand_lo, hi = a.cand_hi;
+  uint32_t* ucnt = reinterpret_cast<uint32_t*>(smem_sel);     // [S]
+  __shared__ SelShared<T, NI> sh;
+  const int seg = blockIdx.x, S = a.S;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int B = max(0, a.keep_a_hi - a.keep_a_lo) + max(0, a.keep_b_hi - a.keep_b_lo) + a.k_exact + a.k_lsh;
-  // flag: 0 candidate, 1 kept, 2 excluded
-  for (int j = threadIdx.x; j < S; j += kSelThreads) {
-    ukey[j] = orderable_f32(a.s_exact[(size_t)seg * S + j]);
-    ucnt[j] = a.counts[(size_t)seg * S + j];
-    const bool kept = (j >= a.keep_a_lo && j < a.keep_a_hi) || (j >= a.keep_b_lo && j < a.keep_b_hi);
-    flag[j] = kept ? 1 : ((j >= a.excl_lo && j < a.excl_hi) ? 2 : 0);
+  const float* s_seg = a.s_exact + (size_t)seg * S;
+  const uint32_t* c_seg = a.counts + (size_t)seg * S;
+  uint32_t v[NI], cand = 0, kept = 0;
+  {
+    float x[NI];
+    uint32_t n[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int j = i * T + (int)threadIdx.x;
+      x[i] = j < S ? s_seg[j] : 0.f;
+      n[i] = j < S ? c_seg[j] : 0u;
+    }
+    for (int i = threadIdx.x; i < kSelBins; i += T) sh.hist[i] = 0;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int j = i * T + (int)threadIdx.x;
+      v[i] = orderable_f32(x[i]);
+      if (j < S) {
+        ucnt[j] = n[i];
+        const bool keep = (j >= a.keep_a_lo && j < a.keep_a_hi) || (j >= a.keep_b_lo && j < a.keep_b_hi);
+        if (keep) kept |= 1u << i;
+        else if (!(j >= a.excl_lo && j < a.excl_hi)) cand |= 1u << i;
+      }
+    }
   }
-  __syncthreads();
   if (a.has_fix) {          // exact signs first: the corrections reach the shared-memory counts as well
-    signfix_segment(a.fix, seg, (int)(threadIdx.x >> 3), kSelThreads >> 3, ucnt);
+    __syncthreads();
+    signfix_segment(a.fix, seg, (int)(threadIdx.x >> 3), T >> 3, ucnt);
     __syncthreads();
   }
-  mark_topk(ukey, flag, lo, hi, a.k_exact, 24, hist, misc, warp_sums);            // K_exact
-  mark_topk(ucnt, flag, lo, hi, a.k_lsh, a.count_top_shift, hist, misc, warp_sums);  // K_lsh from the residual
+  // the candidates' range of scores and of counts
+  uint32_t lo = 0xffffffffu, hi = 0u, clo = 0xffffffffu, chi = 0u;
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    if ((cand >> i) & 1u) {
+      const uint32_t n = ucnt[i * T + (int)threadIdx.x];
+      lo = min(lo, v[i]); hi = max(hi, v[i]);
+      clo = min(clo, n); chi = max(chi, n);
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo); hi = __reduce_max_sync(0xffffffffu, hi);
+  clo = __reduce_min_sync(0xffffffffu, clo); chi = __reduce_max_sync(0xffffffffu, chi);
+  if (lane == 0) { sh.range[0][warp] = lo; sh.range[1][warp] = hi; sh.range[2][warp] = clo; sh.range[3][warp] = chi; }
+  __syncthreads();
+  {
+    const int w = lane & (T / 32 - 1);
+    lo = __reduce_min_sync(0xffffffffu, sh.range[0][w]); hi = __reduce_max_sync(0xffffffffu, sh.range[1][w]);
+    clo = __reduce_min_sync(0xffffffffu, sh.range[2][w]); chi = __reduce_max_sync(0xffffffffu, sh.range[3][w]);
+  }
+  take_topk<T, NI>(v, cand, kept, a.k_exact, lo, hi, sh);            // K_exact
+  if (a.k_lsh > 0) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int j = i * T + (int)threadIdx.x;
+      v[i] = j < S ? ucnt[j] : 0u;
+    }
+    take_topk<T, NI>(v, cand, kept, a.k_lsh, clo, chi, sh);          // K_lsh from the residual
+  }
   // ordered compaction of all kept indices
-  const int per = (S + kSelThreads - 1) / kSelThreads;
-  const int j0 = threadIdx.x * per, j1 = min(S, j0 + per);
-  int cnt = 0;
-  for (int j = j0; j < j1; ++j) cnt += flag[j] == 1;
-  int total;
-  int out = block_exclusive_scan(cnt, warp_sums, total);
-  for (int j = j0; j < j1; ++j)
-    if (flag[j] == 1) { if (out < B) a.idx[(size_t)seg * B + out] = j; ++out; }
+  const int rank0 = ordered_ranks<T, NI>(kept, sh.before[1]);
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    const bool keep = (kept >> i) & 1u;
+    const uint32_t row = __ballot_sync(0xffffffffu, keep);
+    const int out = __shfl_sync(0xffffffffu, rank0, i) + __popc(row & ((1u << lane) - 1u));
+    if (keep && out < B) a.idx[(size_t)seg * B + out] = i * T + (int)threadIdx.x;
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
