@@ -393,8 +393,8 @@ __device__ __forceinline__ bool score_epilogue(const StreamArgs& a, const EpiCtx
       if (a.lse_flags) {
         // the log-sum-exp pass may still be running: wait for the flags of this segment's partials
         bool ready = true;
-        if (e.lane < n_used)
-          ready = wait_flag_equals(a.lse_flags + (size_t)r.c.seg * a.n_slot + e.lane, a.lse_epoch,
+        for (int s2 = e.lane; s2 < n_used && ready; s2 += 32)    // few long segments: more CTAs per segment than lanes
+          ready = wait_flag_equals(a.lse_flags + (size_t)r.c.seg * a.n_slot + s2, a.lse_epoch,
                                    a.poll_ns == 0 ? a.polls : kMaxFlagPolls);
         if (!__all_sync(0xffffffffu, ready)) return false;
       }
