@@ -58,6 +58,7 @@ __host__ __device__ constexpr int proj_acc_stride(int kbits, int tc) { return (k
 __host__ __device__ constexpr int proj_num_acc(int kbits, int tc) {
   return 512 / proj_acc_stride(kbits, tc) < kMaxAcc ? 512 / proj_acc_stride(kbits, tc) : kMaxAcc;
 }
+constexpr int kLseBatch = 8;                  // log-sum-exp partials of a column fetched at a time
 constexpr int kMaxStreamCtas = 256;            // upper bound of the persistent grid (slot arithmetic)
 constexpr int kPolyPairsOf32 = 10;             // of every 32 column pairs, this many take 2^x on the FMA pipe
 
@@ -399,21 +400,41 @@ __device__ __forceinline__ bool score_epilogue(const StreamArgs& a, const EpiCtx
         if (!__all_sync(0xffffffffu, ready)) return false;
       }
       __syncwarp();
+      // Every partial is a round trip to L2 of about 0.7 us: kLseBatch of them are in flight at a time, for
+      // all of the lane's columns (one after the other, a call whose segments are shared by 19 CTAs spent
+      // 7 us here per CTA).
+      constexpr int NH = (NC + 31) / 32;
+      float mx[NH], sum[NH];
 #pragma unroll
-      for (int half = 0; half < (NC + 31) / 32; ++half) {
+      for (int half = 0; half < NH; ++half) { mx[half] = -INFINITY; sum[half] = 0.f; }
+      const float2* p = a.lse_part + (size_t)r.c.seg * a.n_slot * a.GW + c0 + e.lane;
+      for (int s0 = 0; s0 < n_used; s0 += kLseBatch) {
+        float2 pe[NH][kLseBatch];
+#pragma unroll
+        for (int i = 0; i < kLseBatch; ++i)
+#pragma unroll
+          for (int half = 0; half < NH; ++half)
+            pe[half][i] = (s0 + i < n_used && e.lane + 32 * half < NC) ? __ldcg(p + (size_t)(s0 + i) * a.GW + 32 * half)
+                                                                       : make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int half = 0; half < NH; ++half) {
+          float m2 = mx[half];
+#pragma unroll
+          for (int i = 0; i < kLseBatch; ++i) m2 = fmaxf(m2, pe[half][i].x);
+          if (m2 == -INFINITY) continue;
+          if (s0 > 0) sum[half] *= exp2f(mx[half] - m2);
+#pragma unroll
+          for (int i = 0; i < kLseBatch; ++i)
+            if (pe[half][i].x != -INFINITY) sum[half] += pe[half][i].y * exp2f(pe[half][i].x - m2);
+          mx[half] = m2;
+        }
+      }
+#pragma unroll
+      for (int half = 0; half < NH; ++half) {
         const int j = e.lane + 32 * half;
         if (j < NC) {
-          const int qq = c0 + j;
-          const float2* p = a.lse_part + (size_t)r.c.seg * a.n_slot * a.GW + qq;
-          float mx = -INFINITY;
-          for (int s2 = 0; s2 < n_used; ++s2) mx = fmaxf(mx, __ldcg(p + (size_t)s2 * a.GW).x);
-          float sum = 0.f;
-          for (int s2 = 0; s2 < n_used; ++s2) {
-            const float2 pe = __ldcg(p + (size_t)s2 * a.GW);
-            if (pe.x != -INFINITY) sum += pe.y * exp2f(pe.x - mx);
-          }
-          const float lse = mx + log2f(sum);
-          if (r.c.tib == 0 && e.quarter == 0) a.lse2[(size_t)r.c.seg * a.lse2_stride + a.lse2_off + qq] = lse;
+          const float lse = mx[half] + log2f(sum[half]);
+          if (r.c.tib == 0 && e.quarter == 0) a.lse2[(size_t)r.c.seg * a.lse2_stride + a.lse2_off + c0 + j] = lse;
           lw[j] = -lse;
         }
       }
