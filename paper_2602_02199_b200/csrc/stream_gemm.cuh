@@ -776,17 +776,18 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
       const uint32_t stat_lo = umma_sdesc_lo(sm_stat);
       const uint32_t stat_atom_lo = stat_atom_bytes >> 4;
       TileCursor c = cursor_at(x_begin, a);
-      bool new_group = true, need_stat = false;
+      bool new_group = true;
       uint32_t gen = 0, it = 0, last_use = 0;
       int last_acc = -1;
       for (long long x = x_begin; x < x_end; ++x, ++it) {
-        if (new_group) { ++gen; need_stat = true; }   // stationary operand number `gen` serves this tile
+        if (new_group) {
+          // every stationary operand in turn, also one that serves no tile of this warp: a parity tells
+          // only the last two phases apart
+          ok = mbar_wait_spin(bar_stat, gen & 1, a.polls, a.poll_ns);
+          if (!ok) break;
+          ++gen;
+        }
         if (it % kMmaWarps == mine) {
-          if (need_stat) {
-            ok = mbar_wait_spin(bar_stat, (gen - 1) & 1, a.polls, a.poll_ns);
-            if (!ok) break;
-            need_stat = false;
-          }
           const uint32_t s = it % kStages;
           const uint32_t acc = it % NACC, use = it / NACC;
           if (use > 0) ok = mbar_wait_spin(bar_tempty + 8 * acc, (use - 1) & 1, a.polls, a.poll_ns);

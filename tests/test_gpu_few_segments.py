@@ -31,3 +31,20 @@ def test_every_partial_is_waited_for(n_kv_heads, block_size):
         assert (total - 1).abs().max().item() < 1e-4
         want = Bn.laser_kv_window_scores(k, q, block_size, 1)
         assert (s.view_as(want) - want).abs().max().item() <= 1e-5 * want.abs().max().item()
+
+
+@pytest.mark.parametrize("block_size", [64, 128])
+def test_every_stationary_operand_is_waited_for(block_size):
+    """Blocks of one tile, one block per head, more heads than SMs: the stationary operand changes with
+    every tile and each issuing warp works on every second one of them."""
+    import torch
+    from paper_2602_02199_b200 import binding as Bn
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    batch, n_kv_heads, group, window = 100, 8, 4, 32
+    for i in range(4):
+        q = torch.randn(batch, n_kv_heads * group, window, 128, generator=gen, device="cuda").bfloat16()
+        k = torch.randn(batch, n_kv_heads, block_size, 128, generator=gen, device="cuda").bfloat16()
+        s = Bn.laser_kv_window_scores(k, q, block_size, 1)[:, :, 0]
+        logits = torch.einsum("bhgd,bhkd->bhgk", q.double().view(batch, n_kv_heads, group * window, 128), k.double())
+        want = torch.softmax(logits / 128 ** 0.5, dim=-1).sum(2)
+        assert (s.double() - want).abs().max().item() <= 1e-5 * want.abs().max().item()
