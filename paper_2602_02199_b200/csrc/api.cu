@@ -245,6 +245,18 @@ laser_kv_status_t derive(const laser_kv_config_t* c, Derived* d) {
   return LASER_KV_OK;
 }
 
+// Lists of doubtful signs, one per CTA of the projection pass: when `grid` CTAs split the tiles of `nseg`
+// equally long segments times `n_chunks` chunks into equal contiguous slices, a slice meets at most
+// ceil(n_chunks * nseg / grid) + 1 segments, with `fix_cap` items each.
+size_t fix_list_items(int fix_cap, int n_chunks, size_t nseg, int grid) {
+  const size_t met = ((size_t)n_chunks * nseg + grid - 1) / grid + 1;
+  return (size_t)fix_cap * (met < nseg ? met : nseg);
+}
+// Items that hold the lists of any launch over at most `nseg` segments, whatever the grid.
+size_t fix_list_total(int fix_cap, int n_chunks, size_t nseg) {
+  return (size_t)fix_cap * ((size_t)n_chunks * nseg + 2 * (size_t)kMaxStreamCtas);
+}
+
 void carve_ws(const laser_kv_config_t* c, const Derived& d, Carve* v) {
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
@@ -261,7 +273,7 @@ void carve_ws(const laser_kv_config_t* c, const Derived& d, Carve* v) {
   v->counts = take(nseg * S * 4 + 16);     // cleared in 16-byte units
   v->idx = take(nseg * (size_t)(d.B > 0 ? d.B : 1) * 4);
   v->fix_counts = take(nseg * sizeof(int));
-  v->fix_items = take(nseg * (size_t)d.fix_cap * sizeof(int4));
+  v->fix_items = take(fix_list_total(d.fix_cap, d.n_chunks, nseg) * sizeof(int4));
   v->key_buckets = take(c->debug ? nseg * S * d.Lp * 2 : 0);
   v->padP = take((d.Kp != c->lsh_bits || d.Lp != c->lsh_tables) ? (size_t)d.Kp * d.Lp * kHeadDim * 2 : 0);
   v->total = off;
@@ -707,6 +719,8 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
   sa.scale_log2e = d.scale * 1.4426950408889634f;
   sa.lse_part = lse_part; sa.lse2 = lse2; sa.s_exact = s_exact; sa.counts = counts; sa.hist = hist;
   sa.key_buckets = key_buckets; sa.fix_items = fix_items; sa.fix_count = fix_counts; sa.fix_cap = d.fix_cap;
+  sa.K = K0; sa.ks_b = kv_strides[0]; sa.ks_h = kv_strides[1]; sa.ks_t = kv_strides[2]; sa.P = h->P;
+  sa.n_changed = ctrl + 2; sa.n_total = ctrl + 1;
   sa.status = ctrl;
   sa.polls = h->handoff_polls ? h->handoff_polls : kMaxPolls;
   sa.poll_ns = h->handoff_polls ? 0u : kPollHintNs;
@@ -774,17 +788,16 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     const uint32_t smem = stream_smem_bytes(kProj, a3.stat_rows_alloc, d.TC * (2 << d.Kp));
     a3.overlap_prev = (need_exact && !h->profiling) ? 1 : 0;     // beside the tail of the score pass
     a3.end_wait = a3.overlap_prev;                                // the selection kernel follows both
-    LKV_CUDA(launch_proj(d.Kp, d.TC, mapK, h->mapP, a3, stream_grid(a3.n_tiles, h->num_sms), smem, st),
+    const int grid = stream_grid(a3.n_tiles, h->num_sms);
+    a3.fix_list = (int)fix_list_items(d.fix_cap, d.n_chunks, (size_t)nseg, grid);
+    LKV_CUDA(launch_proj(d.Kp, d.TC, mapK, h->mapP, a3, grid, smem, st),
              "projection pass");
   }
   mark();
-  // 5. exact signs where the tensor-core projection was too close to zero (every segment's CTA
-  //    settles its own list first), then the two-stage top-k
+  // 5. two-stage top-k
   {
     SelectArgs sel{s_exact, counts, idx, S_len, g.k_exact, g.k_lsh, g.keep_a_lo, g.keep_a_hi, g.keep_b_lo, g.keep_b_hi,
-                   g.excl_lo, g.excl_hi, need_lsh ? 1 : 0,
-                   SignfixArgs{K0, kv_strides[0], kv_strides[1], kv_strides[2], h->P, hist, counts, key_buckets, fix_items,
-                               fix_counts, d.fix_cap, c.n_kv_heads, nb, S_len, d.Kp, d.Lp, ctrl + 2, S, ctrl + 1}};
+                   g.excl_lo, g.excl_hi};
     const laser_kv_status_t s = launch_select(sel, nseg, h->num_sms, st);
     if (s != LASER_KV_OK) { h->last_error = g_last_error; return s; }
   }
@@ -1333,7 +1346,7 @@ laser_kv_status_t laser_kv_two_stage_topk(const float* s_exact, const uint32_t* 
     return fail(nullptr, LASER_KV_ERR_INVALID_ARG, "two_stage_topk: keep count exceeds the segment");
   if (S > 16384) return fail(nullptr, LASER_KV_ERR_UNSUPPORTED, "two_stage_topk: S > 16384");
   if (2 * anchors + k_exact + k_lsh == 0) return LASER_KV_OK;
-  const SelectArgs sel{s_exact, counts, idx_out, S, k_exact, k_lsh, 0, anchors, S - anchors, S, 0, 0, 0};
+  const SelectArgs sel{s_exact, counts, idx_out, S, k_exact, k_lsh, 0, anchors, S - anchors, S, 0, 0};
   int dev = 0, num_sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
@@ -1589,7 +1602,7 @@ laser_kv_status_t count_geometry(int32_t batch, int32_t n_q_heads, int32_t n_kv_
   cg->off_hist = off; off = align_up(off + bh * lsh_tables * ((size_t)2 << lsh_bits));
   cg->off_qb = off;   off = align_up(off + bh * cg->g.GW * lsh_tables * 2);
   cg->off_fixcnt = off; off = align_up(off + (size_t)cg->g.nseg * sizeof(int));
-  cg->off_fix = off;  off = align_up(off + (size_t)cg->g.nseg * cg->fix_cap * sizeof(int4));
+  cg->off_fix = off;  off = align_up(off + fix_list_total(cg->fix_cap, cg->n_chunks, (size_t)cg->g.nseg) * sizeof(int4));
   cg->total = off;
   return LASER_KV_OK;
 }
@@ -1694,20 +1707,15 @@ laser_kv_status_t laser_kv_collision_counts(const void* K_blk, const void* Q_win
     sa.n_chunks = cg.n_chunks; sa.tables_per_chunk = cg.TC; sa.lsh_bits = lsh_bits; sa.lsh_tables = lsh_tables;
     sa.n_tiles = (long long)g.nseg * g.tiles_in_block * cg.n_chunks;
     sa.stat_rows = cg.TC * lsh_bits; sa.stat_rows_alloc = sa.stat_rows;
-    sa.counts = counts_out; sa.hist = hist; sa.fix_items = fix_items; sa.fix_count = fix_counts; sa.fix_cap = cg.fix_cap;
+    sa.counts = counts_out; sa.hist = hist; sa.fix_items = fix_items; sa.fix_list = (int)fix_list_items(cg.fix_cap, cg.n_chunks, (size_t)g.nseg, stream_grid(sa.n_tiles, num_sms));
+    sa.fix_count = fix_counts; sa.fix_cap = cg.fix_cap;
+    sa.K = static_cast<const uint16_t*>(K_blk); sa.ks_b = kv_strides[0]; sa.ks_h = kv_strides[1]; sa.ks_t = kv_strides[2];
+    sa.P = P; sa.n_changed = ctrl + 2; sa.n_total = ctrl + 1;
     sa.status = ctrl;
     sa.polls = kMaxPolls; sa.poll_ns = kPollHintNs;
     const uint32_t smem = stream_smem_bytes(kProj, sa.stat_rows_alloc, cg.TC * (2 << lsh_bits));
     if ((e = launch_proj(lsh_bits, cg.TC, mapK, mapP, sa, stream_grid(sa.n_tiles, num_sms), smem, st)) != cudaSuccess)
       return fail(nullptr, LASER_KV_ERR_CUDA, "collision_counts: projection pass: %s", cudaGetErrorString(e));
-  }
-  {
-    SignfixArgs fa{static_cast<const uint16_t*>(K_blk), kv_strides[0], kv_strides[1], kv_strides[2], P, hist, counts_out,
-                   nullptr, fix_items, fix_counts, cg.fix_cap, g.H_kv, g.nb, g.S, lsh_bits, lsh_tables, ctrl + 2, g.S, ctrl + 1};
-    signfix_kernel<<<dim3(kSignfixCtasPerSeg, g.nseg), 256, 0, st>>>(fa);
-    g_launches.fetch_add(1);
-    if ((e = cudaGetLastError()) != cudaSuccess)
-      return fail(nullptr, LASER_KV_ERR_CUDA, "collision_counts: signfix_kernel: %s", cudaGetErrorString(e));
   }
   return LASER_KV_OK;
 }

@@ -1,6 +1,4 @@
 // The non-GEMM kernels of the selection path:
-//   signfix_kernel - exact recomputation of key sign bits whose tensor-core projection was too
-//                    close to zero to trust, with the matching correction of the counts.
 //   select_kernel  - Algorithm 1 lines 4-8: two-stage top-k per (sequence, KV head, block) by radix
 //                    selection on registers, ties to the lower index, ascending output.
 //   append_kernel  - gather of the kept K/V rows into the append-only cache (16-byte vectors).
@@ -9,92 +7,6 @@
 #include <stdint.h>
 
 namespace lkv {
-
-__device__ __forceinline__ double bf16_to_f64(uint16_t b) {
-  return static_cast<double>(__uint_as_float(static_cast<uint32_t>(b) << 16));
-}
-
-// ------------------------------------------------------------------------------------------------
-// Exact recomputation of flagged key signs. An item names a key, a table, the provisional bucket
-// code and a mask of the code bits whose projection was too small to trust. Every segment has its
-// own list. Eight lanes per item: for every masked bit the 128-term dot product is formed in fp64
-// (exact bf16 products, sixteen terms per lane, reduction over the eight lanes) and the bit is
-// replaced by its exact sign. If the bucket code changes, the key's count is corrected by
-// hist[new] - hist[old]. The selection kernel runs this for its own segment before it reads the
-// counts; the kernel below serves callers that want the counts alone.
-// ------------------------------------------------------------------------------------------------
-struct SignfixArgs {
-  const uint16_t* Kp;     // keys via strides
-  long long ks_b, ks_h, ks_t;
-  const uint16_t* P;
-  const uint16_t* hist;
-  uint32_t* counts;
-  uint16_t* key_buckets;  // or nullptr
-  const int4* items;      // [seg][cap]: (segment, key, table, code | mask << 16)
-  const int* n_items;     // [seg]
-  int cap;
-  int H_kv, nb, S, K, L;
-  int* n_changed;
-  int S_stride;           // tokens between the first keys of consecutive segments
-  int* n_total;           // sum of the list lengths (reporting)
-};
-
-// The items of segment `seg`, taken by lane group `gid` of `ngroups` (a group = eight consecutive
-// lanes of a warp; all 32 lanes of the warp must call). `smem_counts`, when given, is the calling
-// CTA's copy of the segment's counts and receives the corrections as well.
-__device__ __forceinline__ void signfix_segment(const SignfixArgs& a, int seg, int gid, int ngroups, uint32_t* smem_counts) {
-  const int lane = threadIdx.x & 31;
-  const int sl = lane & 7;                              // lane within the group of eight that shares an item
-  const uint32_t gmask = 0xFFu << (lane & 24);          // the group's lanes
-  const int n = min(a.n_items[seg], a.cap);
-  const int4* items = a.items + (size_t)seg * a.cap;
-  const int t = seg % a.nb;
-  const int h = (seg / a.nb) % a.H_kv;
-  const int b = seg / (a.nb * a.H_kv);
-  for (int it = gid; it < n; it += ngroups) {
-    const int4 item = items[it];
-    const int key = item.y, r = item.z;
-    const uint32_t old_code = (uint32_t)item.w & 0xFFFFu;
-    uint32_t mask = (uint32_t)item.w >> 16;
-    // sixteen key elements per lane
-    const uint16_t* krow = a.Kp + b * a.ks_b + h * a.ks_h + ((long long)t * a.S_stride + key) * a.ks_t + sl * 16;
-    const uint4 ka = *reinterpret_cast<const uint4*>(krow), kb = *reinterpret_cast<const uint4*>(krow + 8);
-    const uint32_t kw[8] = {ka.x, ka.y, ka.z, ka.w, kb.x, kb.y, kb.z, kb.w};
-    uint32_t code = old_code;
-    while (mask) {
-      const int pos = 31 - __clz(mask);          // code bit; hyperplane r*K + (K-1-pos)
-      mask &= ~(1u << pos);
-      const uint16_t* prow = a.P + ((size_t)r * a.K + (a.K - 1 - pos)) * 128 + sl * 16;
-      const uint4 pa = *reinterpret_cast<const uint4*>(prow), pb = *reinterpret_cast<const uint4*>(prow + 8);
-      const uint32_t pw[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
-      double acc0 = 0.0, acc1 = 0.0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        acc0 = fma(bf16_to_f64((uint16_t)(kw[e] & 0xFFFF)), bf16_to_f64((uint16_t)(pw[e] & 0xFFFF)), acc0);
-        acc1 = fma(bf16_to_f64((uint16_t)(kw[e] >> 16)), bf16_to_f64((uint16_t)(pw[e] >> 16)), acc1);
-      }
-      double acc = acc0 + acc1;
-#pragma unroll
-      for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(gmask, acc, off);
-      code = (code & ~(1u << pos)) | ((acc >= 0.0 ? 1u : 0u) << pos);
-    }
-    if (sl == 0 && code != old_code) {
-      const uint16_t* hr = a.hist + ((size_t)(b * a.H_kv + h) * a.L + r) * ((size_t)1 << a.K);
-      const uint32_t delta = (uint32_t)hr[code] - (uint32_t)hr[old_code];
-      atomicAdd(a.counts + (size_t)seg * a.S + key, delta);
-      if (smem_counts) atomicAdd(smem_counts + key, delta);
-      if (a.key_buckets) a.key_buckets[((size_t)seg * a.S + key) * a.L + r] = (uint16_t)code;
-      atomicAdd(a.n_changed, 1);
-    }
-  }
-  if (gid == 0 && sl == 0) atomicAdd(a.n_total, a.n_items[seg]);
-}
-
-constexpr int kSignfixCtasPerSeg = 2;   // CTAs of 256 threads (32 lane groups each) per segment
-
-__global__ void __launch_bounds__(256) signfix_kernel(const SignfixArgs a) {
-  signfix_segment(a, blockIdx.y, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3), (int)((gridDim.x * blockDim.x) >> 3), nullptr);
-}
 
 // ------------------------------------------------------------------------------------------------
 // Two-stage top-k. One CTA of T threads per segment; thread t owns the keys t, t + T, t + 2T, ... and
@@ -105,9 +17,10 @@ __global__ void __launch_bounds__(256) signfix_kernel(const SignfixArgs a) {
 // which they can differ: the first round subtracts the smallest candidate, so that scores that share
 // their exponent bits do not pile up in a few bins (atomics of a warp on one bin go one by one), and
 // the k-th largest of 8192 scores is usually alone in its bin after two rounds, a count after one.
-// A round takes three barriers. Against 8-bit rounds over values and flags in shared memory (whole
-// kernel, doubtful signs included): 512 segments of 4096 keys 62 -> 29 us, 128 of 8192 25.2 -> 20.3 us,
-// 8 of 8192 22.2 -> 16.5 us, 80 of 1864 without signs 7.5 -> 4.7 us.
+// A round takes three barriers. Against 8-bit rounds over values and flags in shared memory (both with the
+// doubtful signs settled in front): 512 segments of 4096 keys 62 -> 29 us, 128 of 8192 25.2 -> 20.3 us, 8 of
+// 8192 22.2 -> 16.5 us; 80 of 1864 without signs 7.5 -> 4.7 us. Since the projection pass settles the
+// signs the first three take 24.7, 12.8 and 10.6 us.
 // ------------------------------------------------------------------------------------------------
 constexpr int kSelBins = 2048;
 constexpr int kSelBinBits = 11;
@@ -266,8 +179,6 @@ struct SelectArgs {
   int S, k_exact, k_lsh;
   int keep_a_lo, keep_a_hi, keep_b_lo, keep_b_hi;   // kept ranges [lo, hi); empty when lo >= hi
   int excl_lo, excl_hi;                             // excluded range
-  int has_fix;              // nonzero: `fix` names the segment lists of doubtful key signs to settle first
-  SignfixArgs fix;
 };
 
 template <int T, int NI>
@@ -302,11 +213,6 @@ __global__ void __launch_bounds__(T, 1024 / T) select_kernel(const SelectArgs a)
         else if (!(j >= a.excl_lo && j < a.excl_hi)) cand |= 1u << i;
       }
     }
-  }
-  if (a.has_fix) {          // exact signs first: the corrections reach the shared-memory counts as well
-    __syncthreads();
-    signfix_segment(a.fix, seg, (int)(threadIdx.x >> 3), T >> 3, ucnt);
-    __syncthreads();
   }
   // the candidates' range of scores and of counts
   uint32_t lo = 0xffffffffu, hi = 0u, clo = 0xffffffffu, chi = 0u;

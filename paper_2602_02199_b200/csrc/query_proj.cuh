@@ -46,27 +46,8 @@ struct QsigArgs {
                            // start while later kernels still run, is held back until all of them have
 };
 
-// <x, y> over 128 bf16 elements in fp64 (every product is exact); 16-byte loads, all in flight at once.
-__device__ __noinline__ double exact_dot128(const uint16_t* x, const uint16_t* y) {
-  uint4 xv[16], yv[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    xv[i] = *reinterpret_cast<const uint4*>(x + 8 * i);
-    yv[i] = *reinterpret_cast<const uint4*>(y + 8 * i);
-  }
-  double acc0 = 0.0, acc1 = 0.0;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const uint32_t xw[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w};
-    const uint32_t yw[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      acc0 = fma(bf16_to_f64((uint16_t)(xw[e] & 0xFFFF)), bf16_to_f64((uint16_t)(yw[e] & 0xFFFF)), acc0);
-      acc1 = fma(bf16_to_f64((uint16_t)(xw[e] >> 16)), bf16_to_f64((uint16_t)(yw[e] >> 16)), acc1);
-    }
-  }
-  return acc0 + acc1;
-}
+// <x, y> over 128 bf16 elements in fp64 (every product is exact).
+__device__ __noinline__ double exact_dot128(const uint16_t* x, const uint16_t* y) { return exact_dot<128>(x, y); }
 
 __host__ __device__ inline uint32_t qsig_smem_bytes(int q_rows_alloc, int kbits) {
   return 2u * q_rows_alloc * 128u + 2u * (kQsigTables * kbits) * 128u + kQsigTables * (4u << kbits) + 64u + 1024u;

@@ -92,9 +92,16 @@ struct StreamArgs {
   uint32_t* counts;        // [seg][S]
   const uint16_t* hist;    // [batch][H_kv][L][2^K]
   uint16_t* key_buckets;   // [seg][S][L] or nullptr
-  int4* fix_items;         // [seg][fix_cap]: (seg, key, table, provisional bucket | doubtful bits << 16)
-  int* fix_count;          // [seg]: items queued for the segment
-  int fix_cap;             // items a segment's list can hold
+  // doubtful key signs (kProj)
+  int4* fix_items;         // [grid][fix_list]: a CTA's items (seg, key, table, provisional bucket | doubtful bits << 16)
+  int fix_list;            // items a CTA's list holds: fix_cap for each segment that its tiles can belong to
+  int* fix_count;          // [seg]: items of the segment
+  int fix_cap;             // a segment with more of them is reported as LASER_KV_ERR_CAPACITY
+  const uint16_t* K;       // keys via strides
+  long long ks_b, ks_h, ks_t;
+  const uint16_t* P;       // hyperplanes
+  int* n_changed;          // items whose bucket changed
+  int* n_total;            // items
   int* status;
   uint32_t polls, poll_ns;     // budget of the hand-off waits: polls, and nanoseconds a poll may suspend
   int overlap_prev;    // launched (with the programmatic-serialization attribute) to start beside the kernel ahead
@@ -193,11 +200,80 @@ __device__ __forceinline__ float sum_exp2(const uint32_t* v, float c2, const flo
   return (acc0.x + acc0.y) + (acc1.x + acc1.y);
 }
 
+// ---- exact signs of doubtful projections ----------------------------------------------------------
+// A projection too close to zero to trust (one in about 20,000) names its key and table in a list of the
+// CTA. The list's counter is a word in shared memory, so that a thread that adds to it goes on after a
+// shared-memory round trip. When the CTA's tiles are done all of its warps settle the list:
+// the doubtful bits of an item are replaced by the signs of fp64 dot products (every bf16 product is
+// exact), and if the bucket code changes the key's count is corrected by hist[new] - hist[old]. An item is
+// a chain of dependent round trips (item, key row and hyperplane, histogram): here 76 groups of eight
+// lanes on every SM share them, where the selection kernel's CTAs, one per segment, took 7 us in front of
+// every selection; select_kernel 25 -> 12.8 us for 128 segments and 16.5 -> 10.6 us for 8, this kernel
+// 4 us longer for 128 segments of 8192 keys and no longer for 8.
+__device__ __forceinline__ double bf16_to_f64(uint16_t b) {
+  return static_cast<double>(__uint_as_float(static_cast<uint32_t>(b) << 16));
+}
+
+// The effects of an item whose exact code is known: one thread.
+template <int KBITS>
+__device__ __forceinline__ void settle_result(const StreamArgs& a, const int4& item, uint32_t code) {
+  const uint32_t old_code = (uint32_t)item.w & 0xFFFFu;
+  if (atomicAdd(a.fix_count + item.x, 1) >= a.fix_cap) record_status(a.status, kStatusCapacity);
+  atomicAdd(a.n_total, 1);
+  if (code == old_code) return;
+  const uint16_t* hr = a.hist + ((size_t)(item.x / a.nb) * a.lsh_tables + item.z) * ((size_t)1 << KBITS);
+  atomicAdd(a.counts + (size_t)item.x * a.S + item.y, (uint32_t)hr[code] - (uint32_t)hr[old_code]);
+  if (a.key_buckets) a.key_buckets[((size_t)item.x * a.S + item.y) * a.lsh_tables + item.z] = (uint16_t)code;
+  atomicAdd(a.n_changed, 1);
+}
+__device__ __forceinline__ const uint16_t* item_key(const StreamArgs& a, const int4& item) {
+  const int t = item.x % a.nb, h = (item.x / a.nb) % a.H_kv, b = item.x / (a.nb * a.H_kv);
+  return a.K + b * a.ks_b + h * a.ks_h + ((long long)t * a.S_stride + item.y) * a.ks_t;
+}
+
+// N elements of x and y (16-byte loads; fp64 accumulation of exact products).
+template <int N>
+__device__ __forceinline__ double exact_dot(const uint16_t* x, const uint16_t* y) {
+  double acc0 = 0.0, acc1 = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; i += 8) {
+    const uint4 xv = *reinterpret_cast<const uint4*>(x + i), yv = *reinterpret_cast<const uint4*>(y + i);
+    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, yw[4] = {yv.x, yv.y, yv.z, yv.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      acc0 = fma(bf16_to_f64((uint16_t)(xw[e] & 0xFFFF)), bf16_to_f64((uint16_t)(yw[e] & 0xFFFF)), acc0);
+      acc1 = fma(bf16_to_f64((uint16_t)(xw[e] >> 16)), bf16_to_f64((uint16_t)(yw[e] >> 16)), acc1);
+    }
+  }
+  return acc0 + acc1;
+}
+
+// Items gid, gid + ngroups, ... of a list of n, eight lanes each (all 32 lanes of a warp call).
+template <int KBITS>
+__device__ __forceinline__ void settle_list(const StreamArgs& a, const int4* items, int n, int gid, int ngroups) {
+  const int lane = threadIdx.x & 31, sl = lane & 7;
+  const uint32_t gmask = 0xFFu << (lane & 24);
+  for (int it = gid; it < n; it += ngroups) {
+    const int4 item = items[it];
+    uint32_t mask = (uint32_t)item.w >> 16, code = (uint32_t)item.w & 0xFFFFu;
+    const uint16_t* key = item_key(a, item) + sl * 16;
+    while (mask) {
+      const int pos = 31 - __clz(mask);
+      mask &= ~(1u << pos);
+      double acc = exact_dot<16>(key, a.P + ((size_t)item.z * KBITS + (KBITS - 1 - pos)) * 128 + sl * 16);
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(gmask, acc, off);
+      code = (code & ~(1u << pos)) | ((acc >= 0.0 ? 1u : 0u) << pos);
+    }
+    if (sl == 0) settle_result<KBITS>(a, item, code);
+  }
+}
+
 // NT consecutive tables of the chunk, starting at table `t_begin` (a multiple of NT), for the
 // calling thread's key: packs the sign bits of each table's K projections into a bucket code,
 // looks the code up in the histogram slice and returns the summed collisions. A table whose
 // smallest |projection| is below 2^-15 of the largest |projection| among the key's first 16
-// hyperplanes of the chunk is queued for an exact recomputation of its signs. All of the thread's
+// hyperplanes of the chunk goes to the CTA's list (`fix_n` items so far) for exact signs. All of the thread's
 // columns are read into registers first and the accumulator buffer is handed back to the MMA warp
 // (arrive on `bar_release`) before the arithmetic starts; the per-table work is branch-free so
 // that the tables interleave. `t_begin` is a run-time value so that the four epilogue groups
@@ -205,7 +281,7 @@ __device__ __forceinline__ float sum_exp2(const uint32_t* v, float c2, const flo
 template <int KBITS, int NT>
 __device__ __forceinline__ uint32_t proj_tables(uint32_t t_acc, uint32_t bar_release, const uint16_t* hist_s,
                                                 const StreamArgs& a, int seg, int key, int table0, int t_begin,
-                                                bool valid) {
+                                                bool valid, int* fix_n) {
   constexpr int NC = NT * KBITS;                               // columns of this thread
   constexpr uint32_t bucket_mask = (1u << KBITS) - 1u;
   uint32_t v[NC];
@@ -258,8 +334,9 @@ __device__ __forceinline__ uint32_t proj_tables(uint32_t t_acc, uint32_t bar_rel
 #pragma unroll
         for (int k = 0; k < KBITS; ++k)
           if (!(fabsf(__uint_as_float(v[t * KBITS + k])) >= tau)) doubt |= 1u << (KBITS - 1 - k);
-        const int slot = atomicAdd(a.fix_count + seg, 1);
-        if (slot < a.fix_cap) a.fix_items[(size_t)seg * a.fix_cap + slot] = make_int4(seg, key, r, (int)(code[t] | (doubt << 16)));
+        const int4 item = make_int4(seg, key, r, (int)(code[t] | (doubt << 16)));
+        const int slot = atomicAdd(fix_n, 1);
+        if (slot < a.fix_list) a.fix_items[(size_t)blockIdx.x * a.fix_list + slot] = item;
         else record_status(a.status, kStatusCapacity);
       }
     }
@@ -276,6 +353,7 @@ struct EpiCtx {
   uint32_t bar_tfull, bar_tempty, bar_stat, bar_stat_free, bar_xa, bar_xb;
   uint8_t* xch_s;              // exchange area
   const uint16_t* hist_s;      // histogram slice (kProj)
+  int* fix_n;                  // items of the CTA's list (kProj)
   uint32_t bar_full, bar_empty, bar_kn;   // kTheory: the epilogue reads the key tile itself
   const uint8_t* stat_s;       // stationary operand, generic pointer (kTheory: query norms)
   const uint8_t* stages_s;     // key-tile ring, generic pointer
@@ -501,7 +579,7 @@ __device__ __forceinline__ bool proj_epilogue(const StreamArgs& a, const EpiCtx&
       tc_fence_after();
       const bool valid = key < a.S;
       const uint32_t partial = proj_tables<KBITS, TQ>(e.t_lane + acc * STRIDE, e.bar_tempty + 8 * acc, e.hist_s, a,
-                                                      r.c.seg, key, table0, e.wg * TQ, valid);
+                                                      r.c.seg, key, table0, e.wg * TQ, valid, e.fix_n);
       if (valid) atomicAdd(cnt + key, partial);
       if (++acc == NACC) { acc = 0; acc_phase ^= 1; }
     }
@@ -636,7 +714,7 @@ template <int MODE, int KBITS, int TC>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, head, batch)
               const __grid_constant__ CUtensorMap map_stat,   // Q: (d, W, H_q, batch) | P: (d, L*K)
-              const StreamArgs a) {
+              const __grid_constant__ StreamArgs a) {
   extern __shared__ uint8_t smem_raw[];
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -692,6 +770,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
       for (int s = 0; s < 2; ++s) { mbar_init(bar_xa + 8 * s, kEpilogueThreads - 128); mbar_init(bar_xb + 8 * s, 128); }
     }
     fence_mbar_init();
+    if (MODE == kProj) *reinterpret_cast<int*>(xch_s) = 0;      // items of the CTA's list of doubtful signs
   }
   if (warp == 1) { tmem_alloc(sm_tmem_slot, kTmemCols); tmem_relinquish(); }
   tc_fence_before();
@@ -844,6 +923,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
     e.bar_xa = bar_xa; e.bar_xb = bar_xb;
     e.xch_s = xch_s;
     e.hist_s = hist_s;
+    e.fix_n = reinterpret_cast<int*>(xch_s);
     e.bar_full = bar_full; e.bar_empty = bar_empty; e.bar_kn = bar_kn;
     e.stat_s = gen_base + (sm_stat - base);
     e.stages_s = gen_base + (sm_stages - base);
@@ -886,11 +966,14 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
   // ---- teardown ----------------------------------------------------------------------------
   tc_fence_before();
   __syncthreads();
-  if (a.end_wait) grid_dependency_wait();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
+  if constexpr (MODE == kProj)
+    settle_list<KBITS>(a, a.fix_items + (size_t)blockIdx.x * a.fix_list, min(*reinterpret_cast<const int*>(xch_s), a.fix_list),
+                       (int)(threadIdx.x >> 3), kStreamThreads >> 3);
+  if (a.end_wait) grid_dependency_wait();
 }
 
 }  // namespace lkv
