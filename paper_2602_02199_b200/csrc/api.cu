@@ -316,31 +316,32 @@ cudaError_t ensure_smem_limit(std::atomic<unsigned long long>& done, Fn* fn, int
   return e;
 }
 
+// Launches a kernel; `beside`: with the programmatic-serialization attribute, so that it may start while the
+// kernel before it in the stream still runs (see ptx.cuh).
+template <typename... Params, typename... Args>
+cudaError_t launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool beside, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = beside ? 1 : 0;
+  const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+  g_launches.fetch_add(1);
+  return le != cudaSuccess ? le : cudaGetLastError();
+}
+
 template <int MODE, int KB, int TCv>
 cudaError_t launch_stream(const CUtensorMap& mk, const CUtensorMap& ms, const StreamArgs& a, int grid,
                           uint32_t smem, cudaStream_t st) {
   static std::atomic<unsigned long long> limit_set{0};   // per instantiation
   const cudaError_t e = ensure_smem_limit(limit_set, stream_kernel<MODE, KB, TCv>, kMaxSmem);
   if (e != cudaSuccess) return e;
-  if (a.overlap_prev) {
-    // may start while the kernel before it in the stream, whose results it does not read, still runs
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kStreamThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, stream_kernel<MODE, KB, TCv>, mk, ms, a);
-    g_launches.fetch_add(1);
-    return le != cudaSuccess ? le : cudaGetLastError();
-  }
-  stream_kernel<MODE, KB, TCv><<<grid, kStreamThreads, smem, st>>>(mk, ms, a);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
+  return launch(stream_kernel<MODE, KB, TCv>, dim3(grid), kStreamThreads, smem, st, a.overlap_prev != 0, mk, ms, a);
 }
 
 cudaError_t launch_proj(int K, int TCv, const CUtensorMap& mk, const CUtensorMap& ms, const StreamArgs& a,
@@ -361,9 +362,7 @@ cudaError_t launch_qsig_t(const CUtensorMap& mq, const CUtensorMap& mp, const Qs
   static std::atomic<unsigned long long> limit_set{0};   // per instantiation
   const cudaError_t e = ensure_smem_limit(limit_set, qsig_kernel<KB>, kMaxSmem);
   if (e != cudaSuccess) return e;
-  qsig_kernel<KB><<<grid, kQsigThreads, smem, st>>>(mq, mp, a);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
+  return launch(qsig_kernel<KB>, grid, kQsigThreads, smem, st, a.overlap_prev != 0, mq, mp, a);
 }
 
 cudaError_t launch_qsig(int K, const CUtensorMap& mq, const CUtensorMap& mp, const QsigArgs& a, dim3 grid, uint32_t smem,
@@ -379,30 +378,28 @@ cudaError_t launch_qsig(int K, const CUtensorMap& mq, const CUtensorMap& mp, con
 }
 
 template <int T, int NI>
-cudaError_t launch_select_t(const SelectArgs& a, int n_seg, cudaStream_t st) {
+cudaError_t launch_select_t(const SelectArgs& a, int n_seg, bool beside, cudaStream_t st) {
   static std::atomic<unsigned long long> limit_set{0};   // per instantiation
   const cudaError_t e = ensure_smem_limit(limit_set, select_kernel<T, NI>, NI * T * 4);
   if (e != cudaSuccess) return e;
-  select_kernel<T, NI><<<n_seg, T, (size_t)a.S * 4, st>>>(a);
-  g_launches.fetch_add(1);
-  return cudaGetLastError();
+  return launch(select_kernel<T, NI>, dim3(n_seg), T, (size_t)a.S * 4, st, beside, a);
 }
 
 // A CTA of 1024 threads per segment: its barriers and its chains of shared-memory round trips set the
 // time, so the fewer keys a thread has the better. Segments of at most 4096 keys that outnumber the
 // SMs go to CTAs of 512 threads, two of which share an SM and hide each other's barriers (512 segments
 // of 4096 keys: 28.9 us; the row counts of the instances are spaced so that at most a third of the rows is empty).
-laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, cudaStream_t st) {
+laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, bool beside, cudaStream_t st) {
   cudaError_t e;
   if (a.S <= 4096 && n_seg > num_sms) {
-    e = a.S <= 1024 ? launch_select_t<512, 2>(a, n_seg, st) : a.S <= 2048 ? launch_select_t<512, 4>(a, n_seg, st)
-                                                                          : launch_select_t<512, 8>(a, n_seg, st);
+    e = a.S <= 1024 ? launch_select_t<512, 2>(a, n_seg, beside, st) : a.S <= 2048 ? launch_select_t<512, 4>(a, n_seg, beside, st)
+                                                                          : launch_select_t<512, 8>(a, n_seg, beside, st);
   } else {
     const int ni = (a.S + 1023) / 1024;
-    e = ni <= 1 ? launch_select_t<1024, 1>(a, n_seg, st) : ni <= 2 ? launch_select_t<1024, 2>(a, n_seg, st)
-      : ni <= 4 ? launch_select_t<1024, 4>(a, n_seg, st) : ni <= 6 ? launch_select_t<1024, 6>(a, n_seg, st)
-      : ni <= 8 ? launch_select_t<1024, 8>(a, n_seg, st) : ni <= 10 ? launch_select_t<1024, 10>(a, n_seg, st)
-      : ni <= 16 ? launch_select_t<1024, 16>(a, n_seg, st) : launch_select_t<1024, 24>(a, n_seg, st);
+    e = ni <= 1 ? launch_select_t<1024, 1>(a, n_seg, beside, st) : ni <= 2 ? launch_select_t<1024, 2>(a, n_seg, beside, st)
+      : ni <= 4 ? launch_select_t<1024, 4>(a, n_seg, beside, st) : ni <= 6 ? launch_select_t<1024, 6>(a, n_seg, beside, st)
+      : ni <= 8 ? launch_select_t<1024, 8>(a, n_seg, beside, st) : ni <= 10 ? launch_select_t<1024, 10>(a, n_seg, beside, st)
+      : ni <= 16 ? launch_select_t<1024, 16>(a, n_seg, beside, st) : launch_select_t<1024, 24>(a, n_seg, beside, st);
   }
   if (e != cudaSuccess) return fail(nullptr, LASER_KV_ERR_CUDA, "select_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
@@ -411,9 +408,7 @@ laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, cud
 laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st) {
   if (a.B <= 0 || n_seg <= 0) return LASER_KV_OK;
   dim3 grid((a.B + kAppendRowsPerCta - 1) / kAppendRowsPerCta, n_seg);
-  append_kernel<<<grid, 256, 0, st>>>(a);
-  g_launches.fetch_add(1);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch(append_kernel, grid, 256, 0, st, false, a);
   if (e != cudaSuccess) return fail(nullptr, LASER_KV_ERR_CUDA, "append_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }
@@ -700,7 +695,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
                   c.n_kv_heads, d.G, d.Wp, d.GWp, q_alloc, d.Lp,
                   reinterpret_cast<uint4*>(counts), ((long long)nseg * S_len + 3) / 4, ctrl + 1, fix_counts, nseg, ctrl,
                   c.lsh_tables, part * d.Wp, part * d.GWp, d.GW, part == 0 ? 1 : 0,
-                  (need_exact && !h->profiling) ? 1 : 0, ctrl + 8};
+                  (need_exact && !h->profiling) ? 1 : 0, ctrl + 8, (part == 0 && !h->profiling) ? 1 : 0};
       dim3 grid(d.Lp / kQsigTables, c.n_kv_heads, c.batch);
       LKV_CUDA(launch_qsig(d.Kp, mapQ, h->mapPq, qa, grid, qsig_smem_bytes(q_alloc, d.Kp), st), "qsig_kernel");
       h->qsig_done_total += grid.x * grid.y * grid.z;
@@ -750,10 +745,11 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     const uint32_t smem = stream_smem_bytes(kScore, a2.stat_rows_alloc, 0);
     // the projection pass reads nothing the score pass writes: it takes each SM as the score pass leaves it
     const bool proj_beside = need_lsh && !h->profiling;
-    a2.release_next = (proj_beside && d.n_qparts == 1) ? 1 : 0;
+    // (without a projection pass the selection follows: it waits for this pass before it reads anything)
+    a2.release_next = (d.n_qparts == 1 && !h->profiling) ? 1 : 0;
     a2.overlap_prev = h->profiling ? 0 : 1;
     if (!h->profiling) { a2.lse_flags = lse_flags; a2.lse_epoch = (int)h->lse_epoch; }
-    if (a2.release_next) { a2.gate_counter = ctrl + 8; a2.gate_target = (int)h->qsig_done_total; }
+    if (a2.release_next && proj_beside) { a2.gate_counter = ctrl + 8; a2.gate_target = (int)h->qsig_done_total; }
     LKV_CUDA((launch_stream<kScore, 0, 0>(mapK, mapQ, a2, base_ctas, smem, st)), "score pass");
     // the remaining parts of a window wider than a pass: their probabilities add to the first part's
     for (int part = 1; part < d.n_qparts; ++part) {
@@ -764,7 +760,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
       b1.stat_rows_alloc = ((d.GWp + 127) / 128) * 128;
       b2.stat_rows_alloc = d.GWp;
       b2.accumulate = 1;
-      b2.release_next = (proj_beside && part == d.n_qparts - 1) ? 1 : 0;
+      b2.release_next = (part == d.n_qparts - 1 && !h->profiling) ? 1 : 0;
       b1.overlap_prev = 0;                                        // follows a score pass: launched the ordinary way
       b1.release_next = h->profiling ? 0 : 1;
       b2.overlap_prev = h->profiling ? 0 : 1;
@@ -773,7 +769,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
         b1.lse_flags = b2.lse_flags = lse_flags;
         b1.lse_epoch = b2.lse_epoch = (int)h->lse_epoch;
       }
-      if (b2.release_next) { b2.gate_counter = ctrl + 8; b2.gate_target = (int)h->qsig_done_total; }
+      if (b2.release_next && proj_beside) { b2.gate_counter = ctrl + 8; b2.gate_target = (int)h->qsig_done_total; }
       LKV_CUDA((launch_stream<kLse, 0, 0>(mapK, mapQ, b1, base_ctas, stream_smem_bytes(kLse, b1.stat_rows_alloc, 0), st)), "lse pass");
       LKV_CUDA((launch_stream<kScore, 0, 0>(mapK, mapQ, b2, base_ctas, smem, st)), "score pass");
     }
@@ -787,6 +783,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     a3.n_tiles = seg_tiles * d.n_chunks;
     const uint32_t smem = stream_smem_bytes(kProj, a3.stat_rows_alloc, d.TC * (2 << d.Kp));
     a3.overlap_prev = (need_exact && !h->profiling) ? 1 : 0;     // beside the tail of the score pass
+    a3.release_next = h->profiling ? 0 : 1;                       // the selection waits for this pass's results
     a3.end_wait = a3.overlap_prev;                                // the selection kernel follows both
     const int grid = stream_grid(a3.n_tiles, h->num_sms);
     a3.fix_list = (int)fix_list_items(d.fix_cap, d.n_chunks, (size_t)nseg, grid);
@@ -794,11 +791,12 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
              "projection pass");
   }
   mark();
-  // 5. two-stage top-k
+  // 5. two-stage top-k, started beside the pass ahead of it. (The append kernel is not started beside the
+  //    selection: with its CTAs resident early four sequences of 128k tokens take 654 instead of 628 us.)
   {
     SelectArgs sel{s_exact, counts, idx, S_len, g.k_exact, g.k_lsh, g.keep_a_lo, g.keep_a_hi, g.keep_b_lo, g.keep_b_hi,
                    g.excl_lo, g.excl_hi};
-    const laser_kv_status_t s = launch_select(sel, nseg, h->num_sms, st);
+    const laser_kv_status_t s = launch_select(sel, nseg, h->num_sms, !h->profiling, st);
     if (s != LASER_KV_OK) { h->last_error = g_last_error; return s; }
   }
   mark();
@@ -1352,7 +1350,7 @@ laser_kv_status_t laser_kv_two_stage_topk(const float* s_exact, const uint32_t* 
   if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
       (e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return fail(nullptr, LASER_KV_ERR_CUDA, "two_stage_topk: device query: %s", cudaGetErrorString(e));
-  return launch_select(sel, n_segments, num_sms, static_cast<cudaStream_t>(stream));
+  return launch_select(sel, n_segments, num_sms, false, static_cast<cudaStream_t>(stream));
 }
 
 // ---- window scores on caller-fed inputs ----------------------------------------------------------

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ptx.cuh"
+
 namespace lkv {
 
 // ------------------------------------------------------------------------------------------------
@@ -192,6 +194,9 @@ __global__ void __launch_bounds__(T, 1024 / T) select_kernel(const SelectArgs a)
   const float* s_seg = a.s_exact + (size_t)seg * S;
   const uint32_t* c_seg = a.counts + (size_t)seg * S;
   uint32_t v[NI], cand = 0, kept = 0;
+  // starts beside the projection pass: only the launch and this are ahead of the wait for its results
+  for (int i = threadIdx.x; i < kSelBins; i += T) sh.hist[i] = 0;
+  grid_dependency_wait();
   {
     float x[NI];
     uint32_t n[NI];
@@ -201,7 +206,6 @@ __global__ void __launch_bounds__(T, 1024 / T) select_kernel(const SelectArgs a)
       x[i] = j < S ? s_seg[j] : 0.f;
       n[i] = j < S ? c_seg[j] : 0u;
     }
-    for (int i = threadIdx.x; i < kSelBins; i += T) sh.hist[i] = 0;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       const int j = i * T + (int)threadIdx.x;
@@ -287,6 +291,7 @@ __device__ __forceinline__ uint4 ld_nc_v4(const void* p) {
 }
 
 __global__ void __launch_bounds__(256, 8) append_kernel(const AppendArgs a) {
+  allow_dependents();                              // the next call's first kernel waits for this one before it does anything
   const int seg = blockIdx.y;                      // (b*H_kv + h)*nb + t
   const int t = seg % a.nb;
   const int bh = seg / a.nb;

@@ -48,6 +48,7 @@ struct QsigArgs {
   int release_next;        // nonzero: the next kernel in the stream was launched to start beside this one
   int* done_counter;       // every CTA adds one when its results are written: the projection pass, which may
                            // start while later kernels still run, is held back until all of them have
+  int overlap_prev;        // nonzero: launched to start beside the kernel ahead in the stream
 };
 
 __host__ __device__ inline uint32_t qsig_smem_bytes(int q_rows_alloc, int kbits) {
@@ -69,8 +70,9 @@ qsig_kernel(const __grid_constant__ CUtensorMap map_q,    // Q: (d, W, H_q, batc
   constexpr uint32_t bucket_mask = nbins - 1u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tg = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  // the log-sum-exp pass that follows needs nothing from this kernel: it may take the SMs this
-  // small grid leaves free (it waits for this kernel only before it ends)
+  // everything before this in the stream is complete, for this kernel and for the one it releases: the
+  // log-sum-exp pass that follows needs nothing from this kernel and takes the SMs this small grid leaves free
+  grid_dependency_wait();
   if (a.release_next) allow_dependents();
   const int nmb = (a.GW + 127) / 128;
   const size_t bh = (size_t)b * a.H_kv + h;
