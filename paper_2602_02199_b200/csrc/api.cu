@@ -405,10 +405,10 @@ laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, boo
   return LASER_KV_OK;
 }
 
-laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st) {
+laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st, bool own_status = false) {
   if (a.B <= 0 || n_seg <= 0) return LASER_KV_OK;
   dim3 grid((a.B + kAppendRowsPerCta - 1) / kAppendRowsPerCta, n_seg);
-  const cudaError_t e = launch(append_kernel, grid, 256, 0, st, false, a);
+  const cudaError_t e = launch(own_status ? append_kernel<true> : append_kernel<false>, grid, 256, 0, st, false, a);
   if (e != cudaSuccess) return fail(nullptr, LASER_KV_ERR_CUDA, "append_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }
@@ -1835,12 +1835,15 @@ laser_kv_status_t laser_kv_gather_append(const void* K_src, const void* V_src, i
       (src_row_stride % 8) || (dst_seg_stride % 8) || (reinterpret_cast<uintptr_t>(status) & 3u))
     return fail(nullptr, LASER_KV_ERR_ALIGNMENT, "gather_append: pointers 16-byte aligned, strides multiples of 8");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int32_t), st);
-  if (e != cudaSuccess) return fail(nullptr, LASER_KV_ERR_CUDA, "gather_append: memset: %s", cudaGetErrorString(e));
+  const bool own_status = n_keep > 0 && (int64_t)n_segments * n_keep <= kAppendOwnStatusMax;
+  if (!own_status) {
+    const cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int32_t), st);
+    if (e != cudaSuccess) return fail(nullptr, LASER_KV_ERR_CUDA, "gather_append: memset: %s", cudaGetErrorString(e));
+  }
   AppendArgs aa{static_cast<const uint16_t*>(K_src), static_cast<const uint16_t*>(V_src), src_seg_stride, 0,
                 src_row_stride, 1, 1, 0, n_keep, idx, static_cast<uint16_t*>(K_dst), static_cast<uint16_t*>(V_dst),
                 pos_out, dst_seg_stride, pos_seg_stride, dst_offset, pos_base, n_src_rows, status};
-  return launch_append(aa, n_segments, st);
+  return launch_append(aa, n_segments, st, own_status);
 }
 
 }  // extern "C"

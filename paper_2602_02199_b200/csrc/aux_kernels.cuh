@@ -280,6 +280,10 @@ struct AppendArgs {
 };
 
 constexpr int kAppendRowsPerCta = 64;
+// Up to this many indices the first CTA looks them all over by itself and stores the status word, so that
+// the caller's word needs no launch of its own to be cleared (one index set gathered head by head: a memset
+// of 1.5 us and its launch in front of every 5 us gather). Above it the scan would outlast the gather.
+constexpr int kAppendOwnStatusMax = 16384;
 constexpr int kAppendBadIndex = 1;   // LASER_KV_ERR_INVALID_ARG
 
 __device__ __forceinline__ uint4 ld_nc_v4(const void* p) {
@@ -290,6 +294,7 @@ __device__ __forceinline__ uint4 ld_nc_v4(const void* p) {
   return v;
 }
 
+template <bool OWN_STATUS>
 __global__ void __launch_bounds__(256, 8) append_kernel(const AppendArgs a) {
   allow_dependents();                              // the next call's first kernel waits for this one before it does anything
   const int seg = blockIdx.y;                      // (b*H_kv + h)*nb + t
@@ -305,7 +310,7 @@ __global__ void __launch_bounds__(256, 8) append_kernel(const AppendArgs a) {
   for (int i = blockIdx.x * kAppendRowsPerCta + (threadIdx.x >> 4); i < i_end; i += 16) {
     const int src = idx ? idx[i] : i;
     if ((unsigned)src >= (unsigned)a.n_src_rows) {          // never read outside the segment
-      if (part == 0) atomicCAS(a.status, 0, kAppendBadIndex);
+      if (!OWN_STATUS && part == 0) atomicCAS(a.status, 0, kAppendBadIndex);
       continue;
     }
     const long long so = src_base + (long long)src * a.ks_t + part * 8;
@@ -315,6 +320,13 @@ __global__ void __launch_bounds__(256, 8) append_kernel(const AppendArgs a) {
     *reinterpret_cast<uint4*>(a.Kc + dof) = kv;
     *reinterpret_cast<uint4*>(a.Vc + dof) = vv;
     if (part == 0) pos[i] = a.pos_base0 + t * a.S_stride + src;
+  }
+  if (OWN_STATUS && blockIdx.x == 0 && blockIdx.y == 0) {
+    const int n = (int)gridDim.y * a.B;
+    int bad = 0;
+    for (int i = threadIdx.x; i < n; i += 256) bad |= (unsigned)a.idx[i] >= (unsigned)a.n_src_rows;
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) *a.status = bad ? kAppendBadIndex : 0;
   }
 }
 

@@ -72,3 +72,25 @@ def test_longest_segment():
     cand = np.concatenate([np.arange(0, a), np.arange(2 * a, a + S - a)])
     want = _want(to_np(dbg.s_exact)[0, 0, 0], to_np(dbg.counts)[0, 0, 0], cand, np.arange(a, 2 * a), k_e, k_l)
     assert (to_np(dbg.idx)[0, 0, 0][:a + b_long] == want).all()
+
+
+@pytest.mark.parametrize("n_seg,keep", [(1, 1), (4, 4096), (5, 4096)])
+def test_gather_status_of_few_and_many_indices(n_seg, keep):
+    """The status word is stored by the gather itself (up to 16384 indices) or cleared before it."""
+    import torch
+    from paper_2602_02199_b200 import binding as Bn
+    rows = 5000
+    src = torch.randn(n_seg, rows, 128, device="cuda").bfloat16()
+    idx = torch.sort(torch.stack([torch.randperm(rows, device="cuda")[:keep] for _ in range(n_seg)]), dim=1)[0].int()
+    k, v = (torch.zeros(n_seg, keep, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    pos = torch.zeros(n_seg, keep, dtype=torch.int32, device="cuda")
+    status = torch.full((1,), 99, dtype=torch.int32, device="cuda")
+    for bad in (False, True, False):
+        use = idx.clone()
+        if bad:
+            use[n_seg - 1, keep - 1] = rows
+        Bn.laser_kv_gather_append(src, src, use, k, v, pos, 0, 0, status)
+        assert int(status) == (Bn.ERR_INVALID_ARG if bad else 0)
+        if not bad:
+            want = torch.gather(src, 1, idx.long()[:, :, None].expand(-1, -1, 128))
+            assert torch.equal(k, want) and torch.equal(v, want) and torch.equal(pos, idx)
