@@ -1174,9 +1174,7 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   static std::atomic<unsigned long long> limit_set{0};
   cudaError_t e = ensure_smem_limit(limit_set, decode_split_kernel, (int)dec_smem_bytes());
   if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel attribute: %s", cudaGetErrorString(e));
-  decode_split_kernel<<<grid, kDecThreads, dec_smem_bytes(), st>>>(mapK, mapV, a);
-  g_launches.fetch_add(1);
-  e = cudaGetLastError();
+  e = launch(decode_split_kernel, grid, kDecThreads, dec_smem_bytes(), st, true, mapK, mapV, a);
   if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }
