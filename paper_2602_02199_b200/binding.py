@@ -200,7 +200,7 @@ def _ptr(t) -> int:
 def _stream_ptr(stream) -> int:
     if stream is None:
         import torch
-        return int(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(getattr(stream, "cuda_stream", stream))
 
 

@@ -84,6 +84,9 @@ struct laser_kv_ctx {
   std::vector<char> lookback_done;      // per layer: laser_kv_lookback_close has run
   struct LayerBudget { int B, anchors, k_exact, k_lsh; };
   std::vector<LayerBudget> budget;      // per layer; the configured budget unless laser_kv_set_layer_budget changed it
+  // decode: a layer's cache as tensor maps, for the length they were encoded for (0: none)
+  struct DecodeMaps { long long len = 0; CUtensorMap k, v; };
+  std::vector<DecodeMaps> decode_maps;
   int last_B = 0;                       // budget of the last select call (debug view)
   std::string last_error;
   bool have_call = false;
@@ -1147,14 +1150,17 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
 
   const size_t layer_off = (size_t)layer * c.batch * c.n_kv_heads * (size_t)d.cap * kHeadDim;
   // the layer's cache as (d, len, H_kv, batch): rows past len read as zeros
-  CUtensorMap mapK, mapV;
-  {
+  if (h->decode_maps.empty()) h->decode_maps.resize(c.n_layers);
+  laser_kv_ctx::DecodeMaps& maps = h->decode_maps[layer];
+  if (maps.len != len) {
     const uint64_t dims[4] = {(uint64_t)kHeadDim, (uint64_t)len, (uint64_t)c.n_kv_heads, (uint64_t)c.batch};
     const uint64_t strides[3] = {(uint64_t)kHeadDim * 2, (uint64_t)d.cap * kHeadDim * 2,
                                  (uint64_t)c.n_kv_heads * d.cap * kHeadDim * 2};
     const uint32_t box[4] = {64, (uint32_t)kDecTile, 1, 1};
-    if (!encode_map(h, &mapK, h->cacheK + layer_off, 4, dims, strides, box)) return LASER_KV_ERR_CUDA;
-    if (!encode_map(h, &mapV, h->cacheV + layer_off, 4, dims, strides, box)) return LASER_KV_ERR_CUDA;
+    maps.len = 0;
+    if (!encode_map(h, &maps.k, h->cacheK + layer_off, 4, dims, strides, box)) return LASER_KV_ERR_CUDA;
+    if (!encode_map(h, &maps.v, h->cacheV + layer_off, 4, dims, strides, box)) return LASER_KV_ERR_CUDA;
+    maps.len = len;
   }
   DecodeArgs a;
   a.Q = static_cast<const uint16_t*>(Q_dec);
@@ -1174,7 +1180,7 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   static std::atomic<unsigned long long> limit_set{0};
   cudaError_t e = ensure_smem_limit(limit_set, decode_split_kernel, (int)dec_smem_bytes());
   if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel attribute: %s", cudaGetErrorString(e));
-  e = launch(decode_split_kernel, grid, kDecThreads, dec_smem_bytes(), st, true, mapK, mapV, a);
+  e = launch(decode_split_kernel, grid, kDecThreads, dec_smem_bytes(), st, true, maps.k, maps.v, a);
   if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }
