@@ -528,6 +528,7 @@ laser_kv_status_t laser_kv_init(const laser_kv_config_t* cfg, const void* hyperp
   h->lookback_done.assign(cfg->n_layers, 0);
   h->budget.assign(cfg->n_layers, laser_kv_ctx::LayerBudget{d.B, d.anchors, d.k_exact, d.k_lsh});
   h->last_B = d.B;
+  h->decode_maps.resize(cfg->n_layers);
   if ((d.Kp != cfg->lsh_bits || d.Lp != cfg->lsh_tables)) {
     // padded copy of the hyperplanes in the workspace (see derive): real bits, then repeats of the
     // table's first hyperplane, then repeats of (padded) table 0
@@ -1150,7 +1151,6 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
 
   const size_t layer_off = (size_t)layer * c.batch * c.n_kv_heads * (size_t)d.cap * kHeadDim;
   // the layer's cache as (d, len, H_kv, batch): rows past len read as zeros
-  if (h->decode_maps.empty()) h->decode_maps.resize(c.n_layers);
   laser_kv_ctx::DecodeMaps& maps = h->decode_maps[layer];
   if (maps.len != len) {
     const uint64_t dims[4] = {(uint64_t)kHeadDim, (uint64_t)len, (uint64_t)c.n_kv_heads, (uint64_t)c.batch};
