@@ -17,8 +17,10 @@
 //                           consumer warps owns 16 rows of every tile: scores S^T = K Q^T,
 //                           numerators relative to the warp's running reference maximum (raised
 //                           only when a score exceeds it by 2^20), O^T += V^T P^T with the
-//                           numerators split into two bf16 terms so that the weights keep
-//                           16 mantissa bits. -> partial (max, sum, G x 128 accumulator) per split.
+//                           numerators split into three bf16 terms so that the weights keep all
+//                           24 bits (two terms: 2.0e-6 instead of 3.4e-7 from fp64 over 1636 entries,
+//                           2.7e-6 instead of 1.6e-6 over 61680; the third costs 1 us of 44 there).
+//                           -> partial (max, sum, G x 128 accumulator) per split.
 //                           The CTA that finishes last for its (sequence, KV head) merges the
 //                           splits' partials in split order and writes the output rows, so the
 //                           whole op is one launch.
@@ -226,18 +228,24 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
         const float p0 = exp2f(x0 - m_a), p1 = exp2f(x1 - m_b), p2 = exp2f(x2 - m_a), p3 = exp2f(x3 - m_b);
         l_a += p0 + p2;
         l_b += p1 + p3;
-        // numerators as two bf16 terms each; transposed they are the B fragments of P^T
+        // numerators as three bf16 terms each, all 24 bits; transposed they are the B fragments of P^T
         const uint32_t h01 = pack_bf16x2(p0, p1), h23 = pack_bf16x2(p2, p3);
         const uint32_t r01 = pack_bf16x2(p0 - __uint_as_float(h01 << 16), p1 - __uint_as_float(h01 & 0xFFFF0000u));
         const uint32_t r23 = pack_bf16x2(p2 - __uint_as_float(h23 << 16), p3 - __uint_as_float(h23 & 0xFFFF0000u));
         const uint32_t bh0 = movmatrix_trans(h01), bh1 = movmatrix_trans(h23);
         const uint32_t bl0 = movmatrix_trans(r01), bl1 = movmatrix_trans(r23);
+        const float q0 = p0 - __uint_as_float(h01 << 16), q1 = p1 - __uint_as_float(h01 & 0xFFFF0000u);
+        const float q2 = p2 - __uint_as_float(h23 << 16), q3 = p3 - __uint_as_float(h23 & 0xFFFF0000u);
+        const uint32_t t01 = pack_bf16x2(q0 - __uint_as_float(r01 << 16), q1 - __uint_as_float(r01 & 0xFFFF0000u));
+        const uint32_t t23 = pack_bf16x2(q2 - __uint_as_float(r23 << 16), q3 - __uint_as_float(r23 & 0xFFFF0000u));
+        const uint32_t bt0 = movmatrix_trans(t01), bt1 = movmatrix_trans(t23);
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
           uint32_t vt[4];
           ldsm_x4_trans(v_tile + dec_swz(warp * 16 + (lane & 7) + 8 * (lane >> 4), 2 * mt + ((lane >> 3) & 1)), vt);
           mma_bf16(o[mt], vt, bh0, bh1);
           mma_bf16(o[mt], vt, bl0, bl1);
+          mma_bf16(o[mt], vt, bt0, bt1);
         }
       }
       __syncwarp();
