@@ -359,6 +359,12 @@ __device__ __forceinline__ float min3_abs(float a, float b, float c) {
   asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+// The same, NaN if any of the three is.
+__device__ __forceinline__ float min3_abs_nan(float a, float b, float c) {
+  float d;
+  asm("min.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
 __device__ __forceinline__ float max3_abs(float a, float b, float c) {
   float d;
   asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));

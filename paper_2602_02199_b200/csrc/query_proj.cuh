@@ -174,7 +174,7 @@ qsig_kernel(const __grid_constant__ CUtensorMap map_q,    // Q: (d, W, H_q, batc
           const uint32_t x0 = v[t * KBITS + k], x1 = v[t * KBITS + k + 1];
           neg = __funnelshift_l(x0, neg, 1);
           neg = __funnelshift_l(x1, neg, 1);
-          mn = min3_abs(__uint_as_float(x0), __uint_as_float(x1), mn);
+          mn = min3_abs_nan(__uint_as_float(x0), __uint_as_float(x1), mn);   // a NaN is doubtful too
         }
         codes[t] = (~neg) & bucket_mask;
         if (!(mn >= tau)) {                         // rare: counted once its signs are settled
