@@ -741,7 +741,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
   const uint32_t bar_tfull = sm_bars + 16 * kStages;   // kMaxAcc: accumulator complete
   const uint32_t bar_tempty = bar_tfull + 8 * kMaxAcc; // kMaxAcc: accumulator copied out by all epilogue threads
   const uint32_t bar_stat = bar_tempty + 8 * kMaxAcc;  // stationary operand landed
-  const uint32_t bar_stat_free = bar_stat + 8;         // stationary operand no longer in use
+  const uint32_t bar_stat_free = bar_stat + 8;         // stationary operand read out by the epilogue threads, seen by the MMA warps
   const uint32_t bar_xa = bar_stat_free + 8;           // 2: mode-specific hand-off, "data written"
   const uint32_t bar_xb = bar_xa + 16;                 // 2: mode-specific hand-off, "data consumed"
   const uint32_t bar_kn = bar_xb + 16;                 // 2: kTheory, key-norm partials of a tile written
@@ -761,7 +761,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
     if (MODE == kTheory) { mbar_init(bar_kn, kEpilogueThreads / 32); mbar_init(bar_kn + 8, kEpilogueThreads / 32); }
     for (int s = 0; s < kMaxAcc; ++s) { mbar_init(bar_tfull + 8 * s, 1); mbar_init(bar_tempty + 8 * s, kEpilogueThreads); }
     mbar_init(bar_stat, 1);
-    mbar_init(bar_stat_free, kEpilogueThreads);
+    mbar_init(bar_stat_free, kEpilogueThreads + kMmaWarps);
     if (MODE == kLse) {
       mbar_init(bar_kn, nmb * 128);                      // column group 0 stored a segment's partial (flag hand-off)
       mbar_init(bar_xa, kEpilogueThreads - nmb * 128);   // column groups 1.. wrote their (max, sum)
@@ -860,8 +860,9 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
       int last_acc = -1;
       for (long long x = x_begin; x < x_end; ++x, ++it) {
         if (new_group) {
-          // every stationary operand in turn, also one that serves no tile of this warp: a parity tells
-          // only the last two phases apart
+          // every stationary operand in turn, also one that serves no tile of this warp: a parity tells only
+          // the last two phases apart, so the producer is held back (arrival below) until both warps have
+          // seen an operand land
           ok = mbar_wait_spin(bar_stat, gen & 1, a.polls, a.poll_ns);
           if (!ok) break;
           ++gen;
@@ -896,6 +897,10 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
           last_use = use;
         }
         new_group = cursor_last_of_group(c, a);
+        if (new_group && x + 1 < x_end) {
+          __syncwarp();                                   // every lane is past the wait for the operand
+          if (lane == 0) mbar_arrive(bar_stat_free);
+        }
         cursor_advance(c, a);
       }
       if (!ok) {
