@@ -248,16 +248,10 @@ laser_kv_status_t derive(const laser_kv_config_t* c, Derived* d) {
   return LASER_KV_OK;
 }
 
-// Lists of doubtful signs, one per CTA of the projection pass: when `grid` CTAs split the tiles of `nseg`
-// equally long segments times `n_chunks` chunks into equal contiguous slices, a slice meets at most
-// ceil(n_chunks * nseg / grid) + 1 segments, with `fix_cap` items each.
-size_t fix_list_items(int fix_cap, int n_chunks, size_t nseg, int grid) {
-  const size_t met = ((size_t)n_chunks * nseg + grid - 1) / grid + 1;
-  return (size_t)fix_cap * (met < nseg ? met : nseg);
-}
-// Items that hold the lists of any launch over at most `nseg` segments, whatever the grid.
-size_t fix_list_total(int fix_cap, int n_chunks, size_t nseg) {
-  return (size_t)fix_cap * ((size_t)n_chunks * nseg + 2 * (size_t)kMaxStreamCtas);
+// Items in each list of doubtful signs when the `grid` CTAs of the projection pass share the room of `nseg` segments.
+int fix_list_items(int fix_cap, size_t nseg, int grid) {
+  const size_t n = (size_t)fix_cap * nseg / (size_t)grid;
+  return (int)(n < (1u << 24) ? n : (1u << 24));
 }
 
 void carve_ws(const laser_kv_config_t* c, const Derived& d, Carve* v) {
@@ -276,7 +270,7 @@ void carve_ws(const laser_kv_config_t* c, const Derived& d, Carve* v) {
   v->counts = take(nseg * S * 4 + 16);     // cleared in 16-byte units
   v->idx = take(nseg * (size_t)(d.B > 0 ? d.B : 1) * 4);
   v->fix_counts = take(nseg * sizeof(int));
-  v->fix_items = take(fix_list_total(d.fix_cap, d.n_chunks, nseg) * sizeof(int4));
+  v->fix_items = take(nseg * (size_t)d.fix_cap * sizeof(int4));
   v->key_buckets = take(c->debug ? nseg * S * d.Lp * 2 : 0);
   v->padP = take((d.Kp != c->lsh_bits || d.Lp != c->lsh_tables) ? (size_t)d.Kp * d.Lp * kHeadDim * 2 : 0);
   v->total = off;
@@ -794,7 +788,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     a3.release_next = h->profiling ? 0 : 1;                       // the selection waits for this pass's results
     a3.end_wait = a3.overlap_prev;                                // the selection kernel follows both
     const int grid = stream_grid(a3.n_tiles, h->num_sms);
-    a3.fix_list = (int)fix_list_items(d.fix_cap, d.n_chunks, (size_t)nseg, grid);
+    a3.fix_list = fix_list_items(d.fix_cap, (size_t)d.nseg_max, grid);
     LKV_CUDA(launch_proj(d.Kp, d.TC, mapK, h->mapP, a3, grid, smem, st),
              "projection pass");
   }
@@ -1608,7 +1602,7 @@ laser_kv_status_t count_geometry(int32_t batch, int32_t n_q_heads, int32_t n_kv_
   cg->off_hist = off; off = align_up(off + bh * lsh_tables * ((size_t)2 << lsh_bits));
   cg->off_qb = off;   off = align_up(off + bh * cg->g.GW * lsh_tables * 2);
   cg->off_fixcnt = off; off = align_up(off + (size_t)cg->g.nseg * sizeof(int));
-  cg->off_fix = off;  off = align_up(off + fix_list_total(cg->fix_cap, cg->n_chunks, (size_t)cg->g.nseg) * sizeof(int4));
+  cg->off_fix = off;  off = align_up(off + (size_t)cg->g.nseg * cg->fix_cap * sizeof(int4));
   cg->total = off;
   return LASER_KV_OK;
 }
@@ -1713,7 +1707,8 @@ laser_kv_status_t laser_kv_collision_counts(const void* K_blk, const void* Q_win
     sa.n_chunks = cg.n_chunks; sa.tables_per_chunk = cg.TC; sa.lsh_bits = lsh_bits; sa.lsh_tables = lsh_tables;
     sa.n_tiles = (long long)g.nseg * g.tiles_in_block * cg.n_chunks;
     sa.stat_rows = cg.TC * lsh_bits; sa.stat_rows_alloc = sa.stat_rows;
-    sa.counts = counts_out; sa.hist = hist; sa.fix_items = fix_items; sa.fix_list = (int)fix_list_items(cg.fix_cap, cg.n_chunks, (size_t)g.nseg, stream_grid(sa.n_tiles, num_sms));
+    sa.counts = counts_out; sa.hist = hist; sa.fix_items = fix_items;
+    sa.fix_list = fix_list_items(cg.fix_cap, (size_t)g.nseg, stream_grid(sa.n_tiles, num_sms));
     sa.fix_count = fix_counts; sa.fix_cap = cg.fix_cap;
     sa.K = static_cast<const uint16_t*>(K_blk); sa.ks_b = kv_strides[0]; sa.ks_h = kv_strides[1]; sa.ks_t = kv_strides[2];
     sa.P = P; sa.n_changed = ctrl + 2; sa.n_total = ctrl + 1;

@@ -94,7 +94,7 @@ struct StreamArgs {
   uint16_t* key_buckets;   // [seg][S][L] or nullptr
   // doubtful key signs (kProj)
   int4* fix_items;         // [grid][fix_list]: a CTA's items (seg, key, table, provisional bucket | doubtful bits << 16)
-  int fix_list;            // items a CTA's list holds: fix_cap for each segment that its tiles can belong to
+  int fix_list;            // items a CTA's list holds: its share of the room for fix_cap items per segment
   int* fix_count;          // [seg]: items of the segment
   int fix_cap;             // a segment with more of them is reported as LASER_KV_ERR_CAPACITY
   const uint16_t* K;       // keys via strides
@@ -210,16 +210,18 @@ __device__ __forceinline__ float sum_exp2(const uint32_t* v, float c2, const flo
 // lanes on every SM share them, where the selection kernel's CTAs, one per segment, took 7 us in front of
 // every selection; select_kernel 25 -> 12.8 us for 128 segments and 16.5 -> 10.6 us for 8, this kernel
 // 4 us longer for 128 segments of 8192 keys and no longer for 8.
+// The lists share the room for as many items as all segments may have, about eight times what is expected. A
+// thread that finds its list full (a run of doubtful keys in a few tiles) settles the table itself: lists of
+// the worst case would take up to 68 times the room.
 __device__ __forceinline__ double bf16_to_f64(uint16_t b) {
   return static_cast<double>(__uint_as_float(static_cast<uint32_t>(b) << 16));
 }
 
-// The effects of an item whose exact code is known: one thread.
+// The effects of an item whose exact code is known: one thread. `before`: items of the segment ahead of it.
 template <int KBITS>
-__device__ __forceinline__ void settle_result(const StreamArgs& a, const int4& item, uint32_t code) {
+__device__ __forceinline__ void settle_result(const StreamArgs& a, const int4& item, uint32_t code, int before) {
   const uint32_t old_code = (uint32_t)item.w & 0xFFFFu;
-  if (atomicAdd(a.fix_count + item.x, 1) >= a.fix_cap) record_status(a.status, kStatusCapacity);
-  atomicAdd(a.n_total, 1);
+  if (before >= a.fix_cap) record_status(a.status, kStatusCapacity);
   if (code == old_code) return;
   const uint16_t* hr = a.hist + ((size_t)(item.x / a.nb) * a.lsh_tables + item.z) * ((size_t)1 << KBITS);
   atomicAdd(a.counts + (size_t)item.x * a.S + item.y, (uint32_t)hr[code] - (uint32_t)hr[old_code]);
@@ -248,6 +250,30 @@ __device__ __forceinline__ double exact_dot(const uint16_t* x, const uint16_t* y
   return acc0 + acc1;
 }
 
+// A table of a key by the calling thread alone, every bit of its code anew. The sums over sixteen elements and the
+// order they are added in are those of the eight lanes below, so that a sign does not depend on who formed it.
+// Not inlined: the copy in the tile loop cost a projection-bound call 2 % of its time.
+template <int KBITS>
+__device__ __noinline__ void settle_alone(const StreamArgs& a, int4 item) {
+  const uint16_t* key = item_key(a, item);
+  const uint16_t* plane = a.P + (size_t)item.z * KBITS * 128;
+  uint32_t code = 0;
+#pragma unroll 1
+  for (int k = 0; k < KBITS; ++k, plane += 128) {
+    double dot = 0.0;
+#pragma unroll 1
+    for (int odd = 0; odd < 2; ++odd) {
+      double half = 0.0;
+#pragma unroll 1
+      for (int s = odd; s < 4; s += 2)
+        half += exact_dot<16>(key + 16 * s, plane + 16 * s) + exact_dot<16>(key + 16 * (s + 4), plane + 16 * (s + 4));
+      dot += half;
+    }
+    code = 2 * code + (dot >= 0.0 ? 1u : 0u);
+  }
+  settle_result<KBITS>(a, item, code, atomicAdd(a.fix_count + item.x, 1));
+}
+
 // Items gid, gid + ngroups, ... of a list of n, eight lanes each (all 32 lanes of a warp call).
 template <int KBITS>
 __device__ __forceinline__ void settle_list(const StreamArgs& a, const int4* items, int n, int gid, int ngroups) {
@@ -256,6 +282,7 @@ __device__ __forceinline__ void settle_list(const StreamArgs& a, const int4* ite
   for (int it = gid; it < n; it += ngroups) {
     const int4 item = items[it];
     uint32_t mask = (uint32_t)item.w >> 16, code = (uint32_t)item.w & 0xFFFFu;
+    const int before = sl == 0 ? atomicAdd(a.fix_count + item.x, 1) : 0;      // under way while the signs are formed
     const uint16_t* key = item_key(a, item) + sl * 16;
     while (mask) {
       const int pos = 31 - __clz(mask);
@@ -265,15 +292,17 @@ __device__ __forceinline__ void settle_list(const StreamArgs& a, const int4* ite
       for (int off = 4; off > 0; off >>= 1) acc += __shfl_xor_sync(gmask, acc, off);
       code = (code & ~(1u << pos)) | ((acc >= 0.0 ? 1u : 0u) << pos);
     }
-    if (sl == 0) settle_result<KBITS>(a, item, code);
+    if (sl == 0) settle_result<KBITS>(a, item, code, before);
   }
 }
 
 // NT consecutive tables of the chunk, starting at table `t_begin` (a multiple of NT), for the
 // calling thread's key: packs the sign bits of each table's K projections into a bucket code,
 // looks the code up in the histogram slice and returns the summed collisions. A table whose
-// smallest |projection| is below 2^-15 of the largest |projection| among the key's first 16
-// hyperplanes of the chunk goes to the CTA's list (`fix_n` items so far) for exact signs. All of the thread's
+// smallest |projection| is below 2^-15 of the largest |projection| among sixteen of the thread's hyperplanes
+// (its first ones; the chunk's first ones where it has fewer) goes to the CTA's list (`fix_n` items so far) for
+// exact signs. The thread's own sixteen need no second load and no registers, which pays for the call of
+// settle_alone: 128k layer 455.0 us without either, 457.7 with the call, 455.0 with both. All of the thread's
 // columns are read into registers first and the accumulator buffer is handed back to the MMA warp
 // (arrive on `bar_release`) before the arithmetic starts; the per-table work is branch-free so
 // that the tables interleave. `t_begin` is a run-time value so that the four epilogue groups
@@ -290,15 +319,16 @@ __device__ __forceinline__ uint32_t proj_tables(uint32_t t_acc, uint32_t bar_rel
 #pragma unroll
   for (int j = 0; j < NC / 32; ++j) tmem_ld_x32(t_col + 32 * j, v + 32 * j);
   if constexpr (NC % 32 != 0) tmem_ld_cols<NC % 32>(t_col + (NC / 32) * 32, v + (NC / 32) * 32);
-  tmem_ld_x16(t_acc, v16);
+  if constexpr (NC < 16) tmem_ld_x16(t_acc, v16);
   tmem_wait_ld();
   reg_fence<NC>(v);
-  reg_fence<16>(v16);
+  if constexpr (NC < 16) reg_fence<16>(v16);
   tc_fence_before();
   mbar_arrive(bar_release);
+  const uint32_t* const scale = NC < 16 ? v16 : v;
   float amax = 0.f;
 #pragma unroll
-  for (int k = 0; k < 16; k += 2) amax = max3_abs(__uint_as_float(v16[k]), __uint_as_float(v16[k + 1]), amax);
+  for (int k = 0; k < 16; k += 2) amax = max3_abs(__uint_as_float(scale[k]), __uint_as_float(scale[k + 1]), amax);
   const float tau = amax * (1.0f / 32768.0f);
   uint32_t code[NT];
   float amin[NT];
@@ -324,7 +354,10 @@ __device__ __forceinline__ uint32_t proj_tables(uint32_t t_acc, uint32_t bar_rel
     partial += hist_g[((uint32_t)t << KBITS) + code[t]];
     lowest = fminf(lowest, amin[t]);
   }
-  if (valid && (a.key_buckets != nullptr || !(lowest >= tau))) {
+  if (__builtin_expect(valid && (a.key_buckets != nullptr || !(lowest >= tau)), 0)) {
+    uint32_t left = 0;                                     // doubtful tables that the CTA's list has no room for
+    uint64_t left_codes = 0;                               // and their codes
+    static_assert(NT * KBITS <= 64, "the codes of a thread's tables in one word");
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
       const int r = table0 + t_begin + t;
@@ -336,9 +369,14 @@ __device__ __forceinline__ uint32_t proj_tables(uint32_t t_acc, uint32_t bar_rel
           if (!(fabsf(__uint_as_float(v[t * KBITS + k])) >= tau)) doubt |= 1u << (KBITS - 1 - k);
         const int4 item = make_int4(seg, key, r, (int)(code[t] | (doubt << 16)));
         const int slot = atomicAdd(fix_n, 1);
-        if (slot < a.fix_list) a.fix_items[(size_t)blockIdx.x * a.fix_list + slot] = item;
-        else record_status(a.status, kStatusCapacity);
+        if (__builtin_expect(slot < a.fix_list, 1)) a.fix_items[(size_t)blockIdx.x * a.fix_list + slot] = item;
+        else { left |= 1u << t; left_codes |= (uint64_t)code[t] << (t * KBITS); }
       }
+    }
+#pragma unroll 1
+    for (; left != 0; left &= left - 1) {
+      const int t = __ffs(left) - 1;
+      settle_alone<KBITS>(a, make_int4(seg, key, table0 + t_begin + t, (int)((uint32_t)(left_codes >> (t * KBITS)) & bucket_mask)));
     }
   }
   return partial;
@@ -975,9 +1013,12 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
-  if constexpr (MODE == kProj)
-    settle_list<KBITS>(a, a.fix_items + (size_t)blockIdx.x * a.fix_list, min(*reinterpret_cast<const int*>(xch_s), a.fix_list),
-                       (int)(threadIdx.x >> 3), kStreamThreads >> 3);
+  if constexpr (MODE == kProj) {
+    const int n = *reinterpret_cast<const int*>(xch_s);
+    if (threadIdx.x == 0 && n > 0) atomicAdd(a.n_total, n);
+    settle_list<KBITS>(a, a.fix_items + (size_t)blockIdx.x * a.fix_list, min(n, a.fix_list), (int)(threadIdx.x >> 3),
+                       kStreamThreads >> 3);
+  }
   if (a.end_wait) grid_dependency_wait();
 }
 

@@ -68,6 +68,26 @@ def test_query_sizes_and_validation():
     assert B.load().laser_kv_status_string(B.ERR_TIMEOUT) == b"device-side wait timed out"
 
 
+@pytest.mark.parametrize("change,most", [
+    (dict(), 17050368), (dict(max_blocks_per_call=1), 2788096),
+    (dict(block_size=1024, window=32, max_blocks=4, max_blocks_per_call=4, lsh_bits=8, lsh_tables=16, context_len=4096), 890368),
+    (dict(block_size=16384, lsh_bits=12, max_blocks=8, max_blocks_per_call=8, lookback=1), 21155584),
+    (dict(batch=4, n_q_heads=28, n_kv_heads=4, block_size=4096, window=32, max_blocks=32, max_blocks_per_call=32, lsh_bits=8,
+          lsh_tables=32, protection_divisor=8), 28288768),
+    (dict(block_size=4096, lsh_bits=6, lsh_tables=128, debug=1, max_blocks_per_call=2), 19216896)])
+def test_workspace_sizes_do_not_grow(change, most):
+    """Callers keep buffers of these sizes: what they were told once stays enough."""
+    base = dict(n_layers=1, block_size=8192, window=64, max_blocks=16, max_blocks_per_call=16, lsh_bits=10, lsh_tables=64,
+                context_len=131072)
+    assert B.laser_kv_query_sizes(_cfg(**{**base, **change}))[1] <= most
+
+
+@pytest.mark.parametrize("shape,most", [((1, 32, 8, 8192, 32, 1, 10, 64), 1442304), ((1, 32, 8, 2048, 64, 8, 10, 32), 918016),
+                                        ((2, 24, 8, 1864, 48, 5, 6, 128), 2045696)])
+def test_collision_count_scratch_does_not_grow(shape, most):
+    assert 0 < B.load().laser_kv_collision_counts_scratch_bytes(*shape) <= most
+
+
 def test_null_and_misaligned_arguments_are_rejected():
     lib = B.load()
     cfg = _cfg()

@@ -44,3 +44,30 @@ def test_run_of_doubtful_keys(n_equal, first):
     want = O.collision_counts(qb, kb)
     assert (counts[first:first + n_equal] == want[first]).all()
     assert (counts[rest] == want[rest]).all()
+
+
+@pytest.mark.parametrize("n_bits,n_tables", [(10, 16), (8, 16), (6, 16), (4, 32), (12, 8), (4, 8), (6, 8)])
+def test_more_doubtful_keys_than_a_ctas_list_holds(n_bits, n_tables):
+    """The segments' lists are shared out over the CTAs of the projection pass: a run of doubtful keys in two
+    tiles is longer than the share of the CTAs that meet it, so most of its items are settled by single threads."""
+    import torch
+    from paper_2602_02199_b200 import binding as Bn
+    H, S, nb, W, G = 2, 1000, 3, 32, 2
+    gen = torch.Generator(device="cuda").manual_seed(n_bits)
+    k = torch.randn(1, H, nb * S, 128, generator=gen, device="cuda")
+    planes = torch.randn(n_tables * n_bits, 128, generator=gen, device="cuda")
+    for row, dim in ((2 * n_bits, 5), (3 * n_bits - 1, 6)):            # first and last bit of table 2
+        planes[row] = 0.0
+        planes[row, dim] = -1.0
+    first = S + 100
+    k[:, 1, first:first + 200, 5:7] = 0.0                              # second head, second block: 200 different keys
+    q = torch.randn(1, H * G, W, 128, generator=gen, device="cuda").bfloat16()
+    k, planes = k.bfloat16(), planes.bfloat16()
+    got, status = Bn.laser_kv_collision_counts(k, q, planes, S, nb, n_bits, n_tables)
+    got = to_np(got).astype(np.int64).reshape(H, nb, S)
+    pb = to_np(planes.view(torch.int16)).view(np.uint16)
+    for h in range(H):
+        qb, _ = O.simhash_buckets(to_np(q[0, h * G:(h + 1) * G].reshape(-1, 128).view(torch.int16)).view(np.uint16), pb, n_bits, n_tables)
+        kb, _ = O.simhash_buckets(to_np(k[0, h].view(torch.int16)).view(np.uint16), pb, n_bits, n_tables)
+        assert (got[h].reshape(-1) == O.collision_counts(qb, kb)).all(), h
+    assert int(status.view(torch.int32)[0]) == 0
