@@ -157,16 +157,18 @@ size_t lse_part_bytes_bound(size_t nseg_max, int GW) {
   return ((size_t)kMaxStreamCtas + 2 * nseg_max) * (size_t)GW * sizeof(float2);
 }
 
-// Largest supported tables-per-chunk for the projection pass: K*TC a multiple of 16 and at most 160
-// columns, L divisible by TC, histogram slice + operands within shared memory. At 160 columns three
-// accumulators fit the TMEM columns and a thread's share of the columns its registers; with 256 (K = 8,
-// 32 tables: two accumulators, spills) four sequences of 128k keys took 757 instead of 706 us.
+// Largest supported tables-per-chunk for the projection pass: K*TC a multiple of 16 and at most 192
+// columns, L divisible by TC, histogram slice + operands within shared memory. A chunk reads all keys, so
+// the wider the better while the epilogue keeps up: 192 columns (6 bits, 32 tables: two accumulators, 48
+// columns a thread, a few spills) against 96, a 128k layer without an exact stage: 128 tables 343 -> 322 us, 64
+// 216 -> 207, 32 166 -> 158; block by block with 32 tables 917 -> 922 for sixteen calls, with 64 977 -> 969.
+// With 256 (8 bits, 32 tables: 64 columns a thread) four sequences of 128k keys took 757 instead of 706 us.
 int pick_tc(int K, int L) {
   const int cands[3] = {32, 16, 8};
   for (int tc : cands) {
     if (L % tc) continue;
     const int n = K * tc;
-    if (n > 160 || (n % 16)) continue;
+    if (n > 192 || (n % 16)) continue;
     const uint32_t smem = stream_smem_bytes(kProj, n, tc * (2 << K));
     if (smem > (uint32_t)kMaxSmem) continue;
     return tc;
@@ -345,7 +347,7 @@ cudaError_t launch_proj(int K, int TCv, const CUtensorMap& mk, const CUtensorMap
                         int grid, uint32_t smem, cudaStream_t st) {
 #define LKV_CASE(KB, T) if (K == KB && TCv == T) return launch_stream<kProj, KB, T>(mk, ms, a, grid, smem, st)
   LKV_CASE(4, 8);  LKV_CASE(4, 16);  LKV_CASE(4, 32);
-  LKV_CASE(6, 8);  LKV_CASE(6, 16);
+  LKV_CASE(6, 8);  LKV_CASE(6, 16);  LKV_CASE(6, 32);
   LKV_CASE(8, 8);  LKV_CASE(8, 16);
   LKV_CASE(10, 8); LKV_CASE(10, 16);
   LKV_CASE(12, 8);

@@ -46,7 +46,7 @@ def test_run_of_doubtful_keys(n_equal, first):
     assert (counts[rest] == want[rest]).all()
 
 
-@pytest.mark.parametrize("n_bits,n_tables", [(10, 16), (8, 16), (6, 16), (4, 32), (12, 8), (4, 8), (6, 8)])
+@pytest.mark.parametrize("n_bits,n_tables", [(10, 16), (8, 16), (6, 16), (4, 32), (12, 8), (4, 8), (6, 8), (6, 32)])
 def test_more_doubtful_keys_than_a_ctas_list_holds(n_bits, n_tables):
     """The segments' lists are shared out over the CTAs of the projection pass: a run of doubtful keys in two
     tiles is longer than the share of the CTAs that meet it, so most of its items are settled by single threads."""
