@@ -389,6 +389,8 @@ cudaError_t launch_select_t(const SelectArgs& a, int n_seg, bool beside, cudaStr
 // SMs go to CTAs of 512 threads, two of which share an SM and hide each other's barriers (512 segments
 // of 4096 keys: 28.9 us; the row counts of the instances are spaced so that at most a third of the rows is empty).
 laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, bool beside, cudaStream_t st) {
+  static_assert(kSelMaxKeys == 24 * 1024, "the largest instance below holds every segment");
+  if (a.S > kSelMaxKeys) return fail(nullptr, LASER_KV_ERR_UNSUPPORTED, "select: segments of more than %d keys", kSelMaxKeys);
   cudaError_t e;
   if (a.S <= 4096 && n_seg > num_sms) {
     e = a.S <= 1024 ? launch_select_t<512, 2>(a, n_seg, beside, st) : a.S <= 2048 ? launch_select_t<512, 4>(a, n_seg, beside, st)
