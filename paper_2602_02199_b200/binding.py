@@ -200,7 +200,9 @@ def _ptr(t) -> int:
 def _stream_ptr(stream) -> int:
     if stream is None:
         import torch
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # the handle without a stream object around it, where this torch offers that
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return int(raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream)
     return int(getattr(stream, "cuda_stream", stream))
 
 

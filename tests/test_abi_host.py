@@ -128,3 +128,13 @@ def test_init_fails_loudly_without_a_gpu():
     st = lib.laser_kv_init(C.byref(cfg), 0x1000, 0x10000, 1 << 40, 0x20000, 1 << 40, C.byref(h))
     assert st == B.ERR_CUDA and not h.value
     assert b"no CPU path" in lib.laser_kv_last_error(None)
+
+
+def test_current_stream_without_torchs_private_function(monkeypatch):
+    import types
+    import torch
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=1234))
+    assert B._stream_ptr(None) == 1234
+    assert B._stream_ptr(types.SimpleNamespace(cuda_stream=77)) == 77
