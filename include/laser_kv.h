@@ -173,10 +173,15 @@ laser_kv_status_t laser_kv_init(const laser_kv_config_t* cfg, const void* hyperp
  * of a sequence is a pass of its own).
  * A handle's workspace serves one call at a time: calls on the same handle must be issued to one
  * stream (or be ordered by the caller); concurrent streams need one handle each.
- * Inside a call some kernels are launched so that they may start before the kernel ahead of them
- * has drained (programmatic stream serialization, where a kernel does not read that kernel's
- * results). Towards everything else on the stream the call behaves as ordinary launches do: its
- * first kernel starts after all earlier work, and work queued after the call starts after all of it.
+ * Inside a call most kernels are launched so that they may start before the kernel ahead of them has
+ * drained (programmatic stream serialization): each waits, before it reads or overwrites anything of a
+ * kernel ahead, until that is in memory. The call's first kernel may be launched beside earlier work on
+ * the stream in the same way; it touches nothing before that work is complete. Work queued after the call
+ * in the ordinary way starts after all of it. The call's last kernel lets a kernel that the caller
+ * launches with the programmatic-serialization attribute start early: such a kernel must execute
+ * griddepcontrol.wait before it reads the cache or overwrites anything the call uses, as the attribute
+ * requires. The same holds for laser_kv_select_tail, laser_kv_lookback_close,
+ * laser_kv_select_block_host, laser_kv_gather_append and laser_kv_decode_attention.
  * Errors: CAPACITY if the cache cannot take n_blocks more blocks or n_blocks exceeds
  * max_blocks_per_call (nothing is launched). */
 laser_kv_status_t laser_kv_select_block(laser_kv_handle_t h, int32_t layer, const void* K_blk,
@@ -459,8 +464,9 @@ laser_kv_status_t laser_kv_gather_append(const void* K_src, const void* V_src,
  *   scratch       : dev, 16-byte aligned, at least laser_kv_decode_attention_scratch_bytes(h) bytes
  *                   (per-chunk partial sums), owned by the caller, reusable after the stream has
  *                   passed the call.
- * Asynchronous on `stream`, ordered after earlier select calls on the same stream. Errors:
- * LASER_KV_ERR_STATE when the layer's cache is empty, LASER_KV_ERR_UNSUPPORTED for more than 8 query
+ * Asynchronous on `stream`, ordered after earlier work on the same stream (the kernel may be launched
+ * beside it and waits for it before it reads anything) and before later work as described at
+ * laser_kv_select_block. Errors: LASER_KV_ERR_STATE when the layer's cache is empty, LASER_KV_ERR_UNSUPPORTED for more than 8 query
  * heads per KV head or more than 1 Mi entries per head, LASER_KV_ERR_CAPACITY for a short scratch. */
 size_t laser_kv_decode_attention_scratch_bytes(laser_kv_handle_t h);
 laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, const void* Q_dec,
