@@ -1,6 +1,7 @@
 """Decode attention at the cache lengths where the number of splits changes its rule (eight tiles, 24
-tiles, three tiles per split), against fp64. The numerators keep 24 bits: what is left is fp32 sums of at
-most 24 terms per accumulator step, a few 1e-7 of the result's norm, and the tensor core's own rounding."""
+tiles, three tiles per split), against fp64. The numerators keep 24 bits: what is left is the rounding of the
+fp32 sums, 1.0e-7 (one tile) to 3.1e-7 of the result's norm over these lengths and six seeds each. Numerators of
+two bf16 terms, 2^-17 off at most, would leave 1.3e-6 to 2.4e-6: the bound of 8e-7 tells the two apart."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -25,4 +26,4 @@ def test_lengths_around_the_split_rule(length, n_kv_heads, group):
     eng.laser_kv_poll_status()
     w = torch.softmax(torch.einsum("bhgd,bhnd->bhgn", q.double().view(1, n_kv_heads, group, 128), k.double()) / 128 ** 0.5, -1)
     want = torch.einsum("bhgn,bhnd->bhgd", w, v.double()).view(1, n_kv_heads * group, 128)
-    assert ((out - want).norm() / want.norm()).item() < 4e-6
+    assert ((out - want).norm() / want.norm()).item() < 8e-7
