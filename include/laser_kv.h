@@ -466,8 +466,9 @@ laser_kv_status_t laser_kv_gather_append(const void* K_src, const void* V_src,
  *                   passed the call.
  * Asynchronous on `stream`, ordered after earlier work on the same stream (the kernel may be launched
  * beside it and waits for it before it reads anything) and before later work as described at
- * laser_kv_select_block. Errors: LASER_KV_ERR_STATE when the layer's cache is empty, LASER_KV_ERR_UNSUPPORTED for more than 8 query
- * heads per KV head or more than 1 Mi entries per head, LASER_KV_ERR_CAPACITY for a short scratch. */
+ * laser_kv_select_block. Errors: LASER_KV_ERR_STATE when the layer's cache is empty,
+ * LASER_KV_ERR_UNSUPPORTED for more than 8 query heads per KV head or more than 1 Mi entries per head,
+ * LASER_KV_ERR_CAPACITY for a short scratch. */
 size_t laser_kv_decode_attention_scratch_bytes(laser_kv_handle_t h);
 laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, const void* Q_dec,
                                             const int64_t q_strides[2], float softmax_scale, float* out,

@@ -416,7 +416,7 @@ laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st,
 
 
 // Splits per (sequence, KV head) of a decode call: as many as fill the GPU's resident CTAs once, but at
-// least three tiles each once there are eight of them: a tile costs a CTA 0.3 us, a split's partials cost
+// most eight of up to 24 tiles and a third of the tiles above: a tile costs a CTA 0.3 us, a split's partials cost
 // the CTA that merges them about as much. us per layer in a captured graph, one tile per split against
 // three: 26 tiles x 8 heads 7.2 / 6.9, 52 x 8 9.2 / 8.2, 103 x 8 11.2 / 10.9, 52 x 4 heads of seven queries
 // 12.0 / 8.0; four tiles 5.0 / 5.3, hence the eight.

@@ -8,7 +8,7 @@
 // per row far below what the memory pipeline needs (a CUDA-core version of the same loop was
 // bound by instruction issue at half the bandwidth). tcgen05 would need M = 128 per instruction
 // and a round trip through TMEM and shared memory for the numerators; nothing is gained when the
-// tensor pipe is busy 14 % of the time as it is.
+// tensor pipe is busy 19 % of the time as it is.
 //
 //   decode_split_kernel   - one CTA per (split of the cache entries, KV head, sequence); the number
 //                           of splits fills the GPU exactly once. A producer warp brings tiles of
@@ -19,7 +19,9 @@
 //                           only when a score exceeds it by 2^20), O^T += V^T P^T with the
 //                           numerators split into three bf16 terms so that the weights keep all
 //                           24 bits (two terms: 2.0e-6 instead of 3.4e-7 from fp64 over 1636 entries,
-//                           2.7e-6 instead of 1.6e-6 over 61680; the third costs 1 us of 44 there).
+//                           2.7e-6 instead of 1.6e-6 over 61680; the third costs 0.4 us of 43 there, 1.7
+//                           of 150 for four such sequences; issuing the MMAs of 2, 4 or 8 row blocks term
+//                           by term, so that they do not wait for one another, changes neither).
 //                           -> partial (max, sum, G x 128 accumulator) per split.
 //                           The CTA that finishes last for its (sequence, KV head) merges the
 //                           splits' partials in split order and writes the output rows, so the

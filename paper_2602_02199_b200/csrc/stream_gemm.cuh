@@ -209,7 +209,7 @@ __device__ __forceinline__ float sum_exp2(const uint32_t* v, float c2, const flo
 // a chain of dependent round trips (item, key row and hyperplane, histogram): here 76 groups of eight
 // lanes on every SM share them, where the selection kernel's CTAs, one per segment, took 7 us in front of
 // every selection; select_kernel 25 -> 12.8 us for 128 segments and 16.5 -> 10.6 us for 8, this kernel
-// 4 us longer for 128 segments of 8192 keys and no longer for 8.
+// 2 us longer for 128 segments of 8192 keys (155.3 -> 157.4 us) and no longer for 8.
 // The lists share the room for as many items as all segments may have, about eight times what is expected. A
 // thread that finds its list full (a run of doubtful keys in a few tiles) settles the table itself: lists of
 // the worst case would take up to 68 times the room.
