@@ -39,12 +39,12 @@ UNIT = "tokens/s"
 # summary of the select call, keyed by (workload, kernel). A missing key means: not captured for
 # this workload, or the kernel has changed since the capture.
 NCU_TRAFFIC_BYTES = {
-    ("llama8b_128k", "stream_kernel<proj>"): 274964480 + 7900416,
-    ("llama8b_128k", "stream_kernel<lse>"): 269273344 + 4132096,
-    ("llama8b_128k", "stream_kernel<score>"): 270247936 + 6919168,
-    ("llama8b_128k", "append_kernel"): 254738688 + 203495168,
-    ("llama8b_128k", "select_kernel"): 17701888,
-    ("llama8b_128k", "decode_split_kernel"): 252766464 + 4244480,
+    ("llama8b_128k", "stream_kernel<proj>"): 281520128 + 3959552,
+    ("llama8b_128k", "stream_kernel<lse>"): 269275648 + 629504,
+    ("llama8b_128k", "stream_kernel<score>"): 270542080 + 3974144,
+    ("llama8b_128k", "append_kernel"): 254752000 + 200093184,
+    ("llama8b_128k", "select_kernel"): 8416768,
+    ("llama8b_128k", "decode_split_kernel"): 252766464 + 512512,
 }
 
 
