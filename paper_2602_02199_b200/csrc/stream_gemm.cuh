@@ -299,10 +299,8 @@ __device__ __forceinline__ void settle_list(const StreamArgs& a, const int4* ite
 // NT consecutive tables of the chunk, starting at table `t_begin` (a multiple of NT), for the
 // calling thread's key: packs the sign bits of each table's K projections into a bucket code,
 // looks the code up in the histogram slice and returns the summed collisions. A table whose
-// smallest |projection| is below 2^-15 of the largest |projection| among sixteen of the thread's hyperplanes
-// (its first ones; the chunk's first ones where it has fewer) goes to the CTA's list (`fix_n` items so far) for
-// exact signs. The thread's own sixteen need no second load and no registers, which pays for the call of
-// settle_alone: 128k layer 455.0 us without either, 457.7 with the call, 455.0 with both. All of the thread's
+// smallest |projection| is below 2^-15 of the largest |projection| among the key's first 16
+// hyperplanes of the chunk goes to the CTA's list (`fix_n` items so far) for exact signs. All of the thread's
 // columns are read into registers first and the accumulator buffer is handed back to the MMA warp
 // (arrive on `bar_release`) before the arithmetic starts; the per-table work is branch-free so
 // that the tables interleave. `t_begin` is a run-time value so that the four epilogue groups
@@ -316,20 +314,22 @@ __device__ __forceinline__ uint32_t proj_tables(uint32_t t_acc, uint32_t bar_rel
   uint32_t v[NC];
   uint32_t v16[16];
   const uint32_t t_col = t_acc + t_begin * KBITS;
+  // the columns of the threshold's scale first: gone from the registers when the thread's own arrive, which pays for
+  // the call of settle_alone below (128k layer 458.6 -> 456.6 us, 455.0 without the call; 32k 102.2 -> 101.7, 101.6)
+  tmem_ld_x16(t_acc, v16);
+  tmem_wait_ld();
+  reg_fence<16>(v16);
 #pragma unroll
   for (int j = 0; j < NC / 32; ++j) tmem_ld_x32(t_col + 32 * j, v + 32 * j);
   if constexpr (NC % 32 != 0) tmem_ld_cols<NC % 32>(t_col + (NC / 32) * 32, v + (NC / 32) * 32);
-  if constexpr (NC < 16) tmem_ld_x16(t_acc, v16);
-  tmem_wait_ld();
-  reg_fence<NC>(v);
-  if constexpr (NC < 16) reg_fence<16>(v16);
-  tc_fence_before();
-  mbar_arrive(bar_release);
-  const uint32_t* const scale = NC < 16 ? v16 : v;
   float amax = 0.f;
 #pragma unroll
-  for (int k = 0; k < 16; k += 2) amax = max3_abs(__uint_as_float(scale[k]), __uint_as_float(scale[k + 1]), amax);
+  for (int k = 0; k < 16; k += 2) amax = max3_abs(__uint_as_float(v16[k]), __uint_as_float(v16[k + 1]), amax);
   const float tau = amax * (1.0f / 32768.0f);
+  tmem_wait_ld();
+  reg_fence<NC>(v);
+  tc_fence_before();
+  mbar_arrive(bar_release);
   uint32_t code[NT];
   float amin[NT];
 #pragma unroll

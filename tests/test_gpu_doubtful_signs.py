@@ -71,3 +71,27 @@ def test_more_doubtful_keys_than_a_ctas_list_holds(n_bits, n_tables):
         kb, _ = O.simhash_buckets(to_np(k[0, h].view(torch.int16)).view(np.uint16), pb, n_bits, n_tables)
         assert (got[h].reshape(-1) == O.collision_counts(qb, kb)).all(), h
     assert int(status.view(torch.int32)[0]) == 0
+
+
+@pytest.mark.parametrize("n_bits,n_tables", [(8, 16), (10, 16), (4, 32), (6, 32)])
+def test_tables_of_zero_hyperplanes(n_bits, n_tables):
+    """The scale of the threshold is that of the chunk's first sixteen hyperplanes for every table of the chunk. Where
+    those are all zero no sign is doubtful, and another table of zero hyperplanes does not fill the list either."""
+    import torch
+    from paper_2602_02199_b200 import binding as Bn
+    H, S, W, G = 2, 1024, 32, 2
+    gen = torch.Generator(device="cuda").manual_seed(60 + n_bits)
+    k = torch.randn(1, H, S, 128, generator=gen, device="cuda").bfloat16()
+    q = torch.randn(1, H * G, W, 128, generator=gen, device="cuda").bfloat16()
+    planes = torch.randn(n_tables, n_bits, 128, generator=gen, device="cuda")
+    planes[:-(-16 // n_bits)] = 0.0
+    planes[n_tables // 4] = 0.0
+    planes = planes.reshape(-1, 128).bfloat16()
+    got, status = Bn.laser_kv_collision_counts(k, q, planes, S, 1, n_bits, n_tables)
+    got, status = to_np(got).astype(np.int64).reshape(H, S), int(status.view(torch.int32)[0])
+    pb = to_np(planes.view(torch.int16)).view(np.uint16)
+    for h in range(H):
+        qb, _ = O.simhash_buckets(to_np(q[0, h * G:(h + 1) * G].reshape(-1, 128).view(torch.int16)).view(np.uint16), pb, n_bits, n_tables)
+        kb, _ = O.simhash_buckets(to_np(k[0, h].view(torch.int16)).view(np.uint16), pb, n_bits, n_tables)
+        assert (got[h] == O.collision_counts(qb, kb)).all(), h
+    assert status == 0
