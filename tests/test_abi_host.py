@@ -134,6 +134,7 @@ def test_current_stream_without_torchs_private_function(monkeypatch):
     import types
     import torch
     monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(B, "_current_stream", None, raising=False)
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=1234))
     assert B._stream_ptr(None) == 1234
