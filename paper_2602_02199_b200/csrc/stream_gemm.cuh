@@ -48,6 +48,7 @@ constexpr int kMmaWarps = 2;
 constexpr int kStreamThreads = 32 * (1 + kMmaWarps) + kEpilogueThreads;
 constexpr int kEpiCols = 64;                   // accumulator columns an epilogue thread holds at most
 constexpr int kXchBytes = 8192;                // exchange area between epilogue warps
+constexpr int kXchScoreBytes = 16384;          // kScore adds the parts of a segment's normalisers [4 groups][4 warps][64 queries]
 constexpr int kXchTheoryBytes = 12288;         // kTheory adds the key-norm partials [2][4 groups][128 keys]
 constexpr int kTmemCols = 512;
 constexpr int kAccStride = 256;                // TMEM columns per accumulator buffer (kLse, kScore: two buffers)
@@ -58,7 +59,8 @@ __host__ __device__ constexpr int proj_acc_stride(int kbits, int tc) { return (k
 __host__ __device__ constexpr int proj_num_acc(int kbits, int tc) {
   return 512 / proj_acc_stride(kbits, tc) < kMaxAcc ? 512 / proj_acc_stride(kbits, tc) : kMaxAcc;
 }
-constexpr int kLseBatch = 8;                  // log-sum-exp partials of a column fetched at a time
+constexpr int kLseSplitAt = 8;                // partials of a segment above which the group's warps share the fetching
+constexpr int kLseBatch = 5;                  // log-sum-exp partials of a column fetched at a time
 constexpr int kMaxStreamCtas = 256;            // upper bound of the persistent grid (slot arithmetic)
 constexpr int kPolyPairsOf32 = 10;             // of every 32 column pairs, this many take 2^x on the FMA pipe
 
@@ -399,7 +401,7 @@ struct EpiCtx {
   int ewarp, wg;               // epilogue warp 0..15, epilogue group 0..3
   uint32_t t_lane;             // TMEM address of the thread's lane, column 0
   long long x_begin, x_end;    // the CTA's slice of the tile sequence
-  uint32_t bar_tfull, bar_tempty, bar_stat, bar_stat_free, bar_xa, bar_xb;
+  uint32_t bar_tfull, bar_tempty, bar_stat, bar_stat_free, bar_xa, bar_xb, bar_norm;
   uint8_t* xch_s;              // exchange area
   const uint16_t* hist_s;      // histogram slice (kProj)
   int* fix_n;                  // items of the CTA's list (kProj)
@@ -511,65 +513,97 @@ __device__ __forceinline__ bool score_epilogue(const StreamArgs& a, const EpiCtx
   float* part = reinterpret_cast<float*>(e.xch_s + 16 * kEpiCols * 4);      // [2 acc][3 groups][128 keys]
   const float c2 = a.scale_log2e;
   uint32_t it = 0;
-  for (long long x = e.x_begin; x < e.x_end;) {
-    const TileRun r = run_at(x, e.x_end, a);
+  uint32_t exchanges = 0;                            // of normalisers' parts so far
+  // segment and first tile of a run, tiles left behind it: the loop over the tiles has no registers to spare
+  int seg, tib, left = (int)(e.x_end - e.x_begin);
+  { const TileCursor c = cursor_at(e.x_begin, a); seg = c.seg; tib = c.tib; }
+  while (left > 0) {
+    int n = min(left, a.tiles_in_block - tib);
+    left -= n;
     if constexpr (NC > 0) {
       // log2-sum-exp2 of this warp's queries from the partials of the CTAs that covered the segment
-      const long long first = (long long)r.c.seg * a.tiles_in_block;
+      const long long first = (long long)seg * a.tiles_in_block;
       const int cf = cta_of_tile(first, a.n_tiles, a.lse_ctas);
       const int n_used = cta_of_tile(first + a.tiles_in_block - 1, a.n_tiles, a.lse_ctas) - cf + 1;
+      // One partial is a round trip to L2 of about 0.7 us, after another one for its flag. Up to kLseSplitAt partials are
+      // fetched by every warp, kLseBatch at a time. More (few segments in the call, each shared by many CTAs) are split over
+      // the group's four warps, which exchange their parts through shared memory: 19 partials, sixteen calls of one block of
+      // 8192 tokens, 958 -> 921 us, calls of two blocks of 4096 276 -> 268.
+      const bool split = n_used > kLseSplitAt;
+      const int first_slot = split ? e.quarter : 0, step = split ? 4 : 1;
+      bool ready = true;
       if (a.lse_flags) {
-        // the log-sum-exp pass may still be running: wait for the flags of this segment's partials
-        bool ready = true;
-        for (int s2 = e.lane; s2 < n_used && ready; s2 += 32)    // few long segments: more CTAs per segment than lanes
-          ready = wait_flag_equals(a.lse_flags + (size_t)r.c.seg * a.n_slot + s2, a.lse_epoch,
+        // the log-sum-exp pass may still be running: wait for the flags of the partials this warp fetches
+        for (int s2 = first_slot + step * e.lane; s2 < n_used && ready; s2 += 32 * step)   // few long segments: more CTAs per segment than lanes
+          ready = wait_flag_equals(a.lse_flags + (size_t)seg * a.n_slot + s2, a.lse_epoch,
                                    a.poll_ns == 0 ? a.polls : kMaxFlagPolls);
         if (!__all_sync(0xffffffffu, ready)) return false;
       }
       __syncwarp();
-      // Every partial is a round trip to L2 of about 0.7 us: kLseBatch of them are in flight at a time, for
-      // all of the lane's columns (one after the other, a call whose segments are shared by 19 CTAs spent
-      // 7 us here per CTA).
       constexpr int NH = (NC + 31) / 32;
       float mx[NH], sum[NH];
 #pragma unroll
       for (int half = 0; half < NH; ++half) { mx[half] = -INFINITY; sum[half] = 0.f; }
-      const float2* p = a.lse_part + (size_t)r.c.seg * a.n_slot * a.GW + c0 + e.lane;
-      for (int s0 = 0; s0 < n_used; s0 += kLseBatch) {
+      const float2* p = a.lse_part + (size_t)seg * a.n_slot * a.GW + c0 + e.lane;
+      for (int s0 = first_slot; s0 < n_used; s0 += step * kLseBatch) {
         float2 pe[NH][kLseBatch];
 #pragma unroll
         for (int i = 0; i < kLseBatch; ++i)
 #pragma unroll
           for (int half = 0; half < NH; ++half)
-            pe[half][i] = (s0 + i < n_used && e.lane + 32 * half < NC) ? __ldcg(p + (size_t)(s0 + i) * a.GW + 32 * half)
-                                                                       : make_float2(-INFINITY, 0.f);
+            pe[half][i] = (s0 + step * i < n_used && e.lane + 32 * half < NC) ? __ldcg(p + (size_t)(s0 + step * i) * a.GW + 32 * half)
+                                                                              : make_float2(-INFINITY, 0.f);
 #pragma unroll
         for (int half = 0; half < NH; ++half) {
           float m2 = mx[half];
 #pragma unroll
           for (int i = 0; i < kLseBatch; ++i) m2 = fmaxf(m2, pe[half][i].x);
           if (m2 == -INFINITY) continue;
-          if (s0 > 0) sum[half] *= exp2f(mx[half] - m2);
+          if (s0 > first_slot) sum[half] *= exp2f(mx[half] - m2);
 #pragma unroll
           for (int i = 0; i < kLseBatch; ++i)
             if (pe[half][i].x != -INFINITY) sum[half] += pe[half][i].y * exp2f(pe[half][i].x - m2);
           mx[half] = m2;
         }
       }
+      if (split) {
+        float2* ex = reinterpret_cast<float2*>(e.xch_s + kXchBytes) + e.wg * 4 * kEpiCols;     // [4 groups][4 warps][64 columns]
+        const uint32_t bar_put = e.bar_norm + 16 * e.wg, bar_got = bar_put + 8;
+        if (!mbar_wait(bar_got, (exchanges + 1) & 1, a.polls, a.poll_ns)) return false;        // passes for the first
+#pragma unroll
+        for (int half = 0; half < NH; ++half) ex[e.quarter * kEpiCols + e.lane + 32 * half] = make_float2(mx[half], sum[half]);
+        __syncwarp();
+        if (e.lane == 0) mbar_arrive(bar_put);
+        if (!mbar_wait(bar_put, exchanges & 1, a.polls, a.poll_ns)) return false;
+#pragma unroll
+        for (int half = 0; half < NH; ++half) {
+          float2 pe[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) pe[i] = ex[i * kEpiCols + e.lane + 32 * half];
+          mx[half] = fmaxf(fmaxf(pe[0].x, pe[1].x), fmaxf(pe[2].x, pe[3].x));
+          sum[half] = 0.f;
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (pe[i].x != -INFINITY) sum[half] += pe[i].y * exp2f(pe[i].x - mx[half]);
+        }
+        __syncwarp();
+        if (e.lane == 0) mbar_arrive(bar_got);
+        ++exchanges;
+      }
 #pragma unroll
       for (int half = 0; half < NH; ++half) {
         const int j = e.lane + 32 * half;
         if (j < NC) {
           const float lse = mx[half] + log2f(sum[half]);
-          if (r.c.tib == 0 && e.quarter == 0) a.lse2[(size_t)r.c.seg * a.lse2_stride + a.lse2_off + c0 + j] = lse;
+          if (tib == 0 && e.quarter == 0) a.lse2[(size_t)seg * a.lse2_stride + a.lse2_off + c0 + j] = lse;
           lw[j] = -lse;
         }
       }
       __syncwarp();
     }
-    float* out = a.s_exact + (size_t)r.c.seg * a.S;
-    int key = r.c.tib * kTileKeys + e.row;
-    for (int j = 0; j < r.ntiles; ++j, ++it, key += kTileKeys) {
+    float* out = a.s_exact + (size_t)seg * a.S;
+    int key = tib * kTileKeys + e.row;
+    for (; n > 0; --n, ++it, key += kTileKeys) {
       const uint32_t acc = it & 1;
       if (!mbar_wait(e.bar_tfull + 8 * acc, (it >> 1) & 1, a.polls, a.poll_ns)) return false;
       tc_fence_after();
@@ -597,8 +631,8 @@ __device__ __forceinline__ bool score_epilogue(const StreamArgs& a, const EpiCtx
         if (key < a.S) out[key] = a.accumulate ? out[key] + tot : tot;
       }
     }
-    x += r.ntiles;
-    if (r.ends_group && x < e.x_end) mbar_arrive(e.bar_stat_free);
+    tib = 0;
+    if (left > 0 && ++seg % a.nb == 0) mbar_arrive(e.bar_stat_free);      // the next segment is another head's
   }
   return true;
 }
@@ -754,8 +788,8 @@ __device__ __forceinline__ bool theory_epilogue(const StreamArgs& a, const EpiCt
 __host__ __device__ inline uint32_t stream_smem_bytes(int mode, int stat_rows_alloc, int hist_bytes) {
   uint32_t b = 2u * stat_rows_alloc * 128u + kStages * kTileBytes;
   if (mode == kProj) b += (hist_bytes + 127u) & ~127u;
-  b += (mode == kTheory) ? kXchTheoryBytes : kXchBytes;    // exchange area: per-warp values, cross-group partials
-  b += 256;          // barriers + TMEM slot
+  b += (mode == kTheory) ? kXchTheoryBytes : (mode == kScore) ? kXchScoreBytes : kXchBytes;    // exchange area: per-warp values, cross-group partials
+  b += 320;          // barriers + TMEM slot
   return b + 1024;   // slack for 1024-byte alignment of the base
 }
 
@@ -790,9 +824,9 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
   const uint32_t sm_hist = cur;
   if (MODE == kProj) cur += (hist_bytes + 127u) & ~127u;
   const uint32_t sm_xch = cur;
-  cur += (MODE == kTheory) ? kXchTheoryBytes : kXchBytes;
+  cur += (MODE == kTheory) ? kXchTheoryBytes : (MODE == kScore) ? kXchScoreBytes : kXchBytes;
   const uint32_t sm_bars = cur;
-  const uint32_t sm_tmem_slot = cur + 192;
+  const uint32_t sm_tmem_slot = cur + 256;
   const uint32_t bar_full = sm_bars;                   // kStages barriers: tile landed
   const uint32_t bar_empty = sm_bars + 8 * kStages;    // kStages barriers: tile consumed by the MMAs
   const uint32_t bar_tfull = sm_bars + 16 * kStages;   // kMaxAcc: accumulator complete
@@ -802,6 +836,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
   const uint32_t bar_xa = bar_stat_free + 8;           // 2: mode-specific hand-off, "data written"
   const uint32_t bar_xb = bar_xa + 16;                 // 2: mode-specific hand-off, "data consumed"
   const uint32_t bar_kn = bar_xb + 16;                 // 2: kTheory, key-norm partials of a tile written
+  const uint32_t bar_norm = bar_kn + 16;               // 2 for each group, kScore: parts of a segment's normalisers written, read
   uint8_t* const gen_base = smem_raw + (base - smem_u32(smem_raw));
   const uint16_t* hist_s = reinterpret_cast<const uint16_t*>(gen_base + (sm_hist - base));
   uint8_t* const xch_s = gen_base + (sm_xch - base);
@@ -826,6 +861,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
     } else {
       for (int s = 0; s < 2; ++s) { mbar_init(bar_xa + 8 * s, kEpilogueThreads - 128); mbar_init(bar_xb + 8 * s, 128); }
     }
+    if (MODE == kScore) for (int s = 0; s < 2 * kEpiGroups; ++s) mbar_init(bar_norm + 8 * s, 4);
     fence_mbar_init();
     if (MODE == kProj) *reinterpret_cast<int*>(xch_s) = 0;      // items of the CTA's list of doubtful signs
   }
@@ -982,7 +1018,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
     e.x_begin = x_begin;
     e.x_end = x_end;
     e.bar_tfull = bar_tfull; e.bar_tempty = bar_tempty; e.bar_stat = bar_stat; e.bar_stat_free = bar_stat_free;
-    e.bar_xa = bar_xa; e.bar_xb = bar_xb;
+    e.bar_xa = bar_xa; e.bar_xb = bar_xb; e.bar_norm = bar_norm;
     e.xch_s = xch_s;
     e.hist_s = hist_s;
     e.fix_n = reinterpret_cast<int*>(xch_s);
