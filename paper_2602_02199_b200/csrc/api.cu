@@ -304,13 +304,14 @@ bool encode_map(laser_kv_ctx* h, CUtensorMap* m, const void* ptr, int rank, cons
 // The dynamic shared-memory limit is an attribute of (kernel, device): set it once per device that
 // the process launches the kernel on. `done` holds one bit per device ordinal below 64.
 template <typename Fn>
-cudaError_t ensure_smem_limit(std::atomic<unsigned long long>& done, Fn* fn, int bytes) {
+cudaError_t ensure_smem_limit(std::atomic<unsigned long long>& done, Fn* fn, int bytes, bool any_cluster = false) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const unsigned long long bit = (dev >= 0 && dev < 64) ? 1ull << dev : 0ull;
   if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && any_cluster) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && bit) done.fetch_or(bit);
   return e;
 }
@@ -318,20 +319,33 @@ cudaError_t ensure_smem_limit(std::atomic<unsigned long long>& done, Fn* fn, int
 // Launches a kernel; `beside`: with the programmatic-serialization attribute, so that it may start while the
 // kernel before it in the stream still runs (see ptx.cuh).
 template <typename... Params, typename... Args>
-cudaError_t launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool beside, Args&&... args) {
+cudaError_t launch_clusters(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool beside, int cluster,
+                            Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
-  cfg.numAttrs = beside ? 1 : 0;
+  if (beside) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
   g_launches.fetch_add(1);
   return le != cudaSuccess ? le : cudaGetLastError();
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool beside, Args&&... args) {
+  return launch_clusters(kernel, grid, threads, smem, st, beside, 1, args...);
 }
 
 template <int MODE, int KB, int TCv>
@@ -453,6 +467,29 @@ void weight_proj_slices(StreamArgs* a, int grid, int qsig_ctas, int abreast) {
   const long long w_less = less * a->w_early / per;
   const long long most = a->w_early * 45ll / 100;
   a->w_late = a->w_early - (int)(w_less < most ? w_less : most);
+}
+
+// Splits per (sequence, KV head) that merge inside a thread-block cluster (0: n_split of them by way of global memory, where
+// a partial goes to memory, is counted there and comes back to the CTA that merges). us per layer in a captured graph, by way of
+// memory against a cluster of at most eight: 8 heads of four queries and 4 tiles 5.2 / 3.5, 13 5.9 / 4.5, 26 7.2 / 6.3, 64 9.3 /
+// 8.5, 103 10.8 / 10.9; 4 heads of seven queries and 26 tiles 7.4 / 5.4. A cluster has to find room on one part of the GPU:
+// up to 256 CTAs in all do (264 of them 10.3 against 10.7, 280 14.3 against 10.8).
+// Longer caches of few heads with many queries: the general path's merge costs as much as its partials are large, a cluster
+// of sixteen reads the cache with fewer CTAs (4 heads of seven queries, 150 tiles 15.5 / 10.4, 512 24.5 / 21.2, 1024
+// 35.1 / 36.2; one head of eight, 512 28.4 / 18.5; 8 heads of four, 80 10.0 / 9.2, 255 16.9 / 16.6, 512 27.0 / 27.4; 4 heads
+// of two, 80 6.9 / 7.2). The inequality is where the two cross, from these and twenty more.
+int decode_cluster(const laser_kv_ctx* h, long long len, int n_split) {
+  const laser_kv_config_t& c = h->cfg;
+  const long long tiles = (len + kDecTile - 1) / kDecTile, heads = (long long)c.batch * c.n_kv_heads;
+  if (tiles <= 64) {
+    long long n = (long long)h->num_sms * kDecCtasPerSm / heads;
+    if (n > 8) n = 8;
+    if (n > tiles) n = tiles;
+    if (n <= 1) return 1;
+    return n * heads <= 256 ? (int)n : 0;
+  }
+  const long long G = c.n_q_heads / c.n_kv_heads;
+  return 16 * heads <= h->num_sms && 3 * (G * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
 }
 
 }  // namespace
@@ -1207,11 +1244,19 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   a.status = reinterpret_cast<int*>(h->ws + h->carve.ctrl);
   a.counters = reinterpret_cast<int*>(h->ws + h->carve.dec_count);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const dim3 grid((unsigned)n_split, (unsigned)c.n_kv_heads, (unsigned)c.batch);
-  static std::atomic<unsigned long long> limit_set{0};
-  cudaError_t e = ensure_smem_limit(limit_set, decode_split_kernel, (int)dec_smem_bytes());
-  if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel attribute: %s", cudaGetErrorString(e));
-  e = launch(decode_split_kernel, grid, kDecThreads, dec_smem_bytes(), st, true, maps.k, maps.v, a);
+  cudaError_t e;
+  const int n_cluster = decode_cluster(h, len, n_split);
+  auto run = [&](auto kernel, std::atomic<unsigned long long>& limit_set, int n, bool any_cluster, int cluster) {
+    a.n_split = n;
+    const cudaError_t le = ensure_smem_limit(limit_set, kernel, (int)dec_smem_bytes(), any_cluster);
+    if (le != cudaSuccess) return le;
+    return launch_clusters(kernel, dim3((unsigned)n, (unsigned)c.n_kv_heads, (unsigned)c.batch), kDecThreads, dec_smem_bytes(), st, true,
+                           cluster, maps.k, maps.v, a);
+  };
+  static std::atomic<unsigned long long> limit0{0}, limit8{0}, limit16{0};
+  if (n_cluster == 0) e = run(decode_split_kernel<0>, limit0, n_split, false, 1);
+  else if (n_cluster <= 8) e = run(decode_split_kernel<8>, limit8, n_cluster, false, n_cluster);
+  else e = run(decode_split_kernel<16>, limit16, n_cluster, true, n_cluster);
   if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }

@@ -18,14 +18,16 @@
 //                           numerators relative to the warp's running reference maximum (raised
 //                           only when a score exceeds it by 2^20), O^T += V^T P^T with the
 //                           numerators split into three bf16 terms so that the weights keep all
-//                           24 bits (two terms: 2.0e-6 instead of 3.4e-7 from fp64 over 1636 entries,
-//                           2.7e-6 instead of 1.6e-6 over 61680; the third costs 0.4 us of 43 there, 1.7
-//                           of 150 for four such sequences; issuing the MMAs of 2, 4 or 8 row blocks term
+//                           24 bits (two terms: 2.0e-6 instead of 3.4e-7 from fp64 over 1636 entries
+//                           when a split had one accumulator; the third costs 0.4 us of 43 over
+//                           61680, 1.7 of 150 for four such sequences; issuing the MMAs of 2, 4 or 8 row blocks term
 //                           by term, so that they do not wait for one another, changes neither).
 //                           -> partial (max, sum, G x 128 accumulator) per split.
-//                           The CTA that finishes last for its (sequence, KV head) merges the
-//                           splits' partials in split order and writes the output rows, so the
-//                           whole op is one launch.
+//                           The splits of a (sequence, KV head) are one thread-block cluster
+//                           where they are few: every CTA forms a share of the output from the
+//                           others' partials in shared memory (see the cluster rule at the
+//                           launch). Otherwise the CTA that finishes last merges the partials, by
+//                           way of global memory, in split order. The whole op is one launch.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -47,6 +49,7 @@ constexpr int kDecMaxGroup = 8;         // query heads per KV head, at most (the
 constexpr int kDecPartFloats = 128 + 4; // per (split, query head): accumulator, reference max, sum, padding to 16 bytes
 constexpr int kDecMaxSplit = 512;
 constexpr float kDecRescaleAt = 20.f;   // log2 units a score may exceed the reference maximum by
+constexpr uint32_t kDecClusterOffset = 20480;   // their partials in shared memory, behind the warps' merge buffer
 constexpr int kDecRedStride = 132;      // floats between heads in the merge buffer (bank spread)
 
 struct DecodeArgs {
@@ -96,9 +99,26 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return y;
 }
 
+// ---- thread-block clusters: the shared memory of the cluster's CTAs ----
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address in CTA `rank` of the cluster that corresponds to a shared-memory address of this CTA.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 // MMA fragment coordinates of a lane: g = lane / 4 (a row of the 16-row operand, a column of B),
 // c = lane % 4 (the pair of columns 2c, 2c+1). Scores come out as S^T[key g (+8)][heads 2c, 2c+1];
 // the accumulators are O^T[dim 16 mt + g (+8)][heads 2c, 2c+1].
+template <int CLUSTER>
 __global__ void __launch_bounds__(kDecThreads, kDecCtasPerSm)
 decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d, len, H_kv, batch), box (64, 64, 1, 1)
                     const __grid_constant__ CUtensorMap map_v,    // cache V, same shape
@@ -137,12 +157,16 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
   grid_dependency_wait();
   allow_dependents();
 
-  float o[8][4];                 // O^T, eight 16-dim row blocks
+  // O^T, eight 16-dim row blocks: of the running tiles, and of those before. The MMAs' own accumulators do not round to nearest;
+  // added up outside them every few tiles, the result over 1636 entries is 1.4e-7 instead of 2.2e-7 from fp64, over 61,680
+  // 2.5e-7 instead of 1.3e-6. (Tile by tile a cache of 61,680 entries takes 1 % longer, short ones no longer.)
+  constexpr int kTilesPerSum = CLUSTER > 0 ? 1 : 4;
+  float o[8][4], o_sum[8][4];
   float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;   // heads 2c and 2c+1
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) o[mt][i] = 0.f;
+    for (int i = 0; i < 4; ++i) o[mt][i] = o_sum[mt][i] = 0.f;
 
   if (warp == kDecWarps) {
     // ---- producer: one lane keeps the ring full -----------------------------------------------------
@@ -225,7 +249,10 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
           m_a = n_a; m_b = n_b;
           l_a *= f_a; l_b *= f_b;
 #pragma unroll
-          for (int mt = 0; mt < 8; ++mt) { o[mt][0] *= f_a; o[mt][1] *= f_b; o[mt][2] *= f_a; o[mt][3] *= f_b; }
+          for (int mt = 0; mt < 8; ++mt) {
+            if (kTilesPerSum > 1) { o[mt][0] *= f_a; o[mt][1] *= f_b; o[mt][2] *= f_a; o[mt][3] *= f_b; }
+            o_sum[mt][0] *= f_a; o_sum[mt][1] *= f_b; o_sum[mt][2] *= f_a; o_sum[mt][3] *= f_b;
+          }
         }
         const float p0 = exp2f(x0 - m_a), p1 = exp2f(x1 - m_b), p2 = exp2f(x2 - m_a), p3 = exp2f(x3 - m_b);
         l_a += p0 + p2;
@@ -252,6 +279,12 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_empty(st));
+      if (kTilesPerSum == 1 || t % kTilesPerSum == kTilesPerSum - 1 || t == n_tiles - 1) {
+#pragma unroll
+        for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) { o_sum[mt][i] += o[mt][i]; o[mt][i] = 0.f; }
+      }
     }
     // the warp's sums over its keys: lanes with equal c hold different keys
 #pragma unroll
@@ -273,13 +306,61 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
     float* dst = red + (warp * 8 + 2 * c) * kDecRedStride;
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) {
-      dst[16 * mt + g] = o[mt][0] * f_a;
-      dst[kDecRedStride + 16 * mt + g] = o[mt][1] * f_b;
-      dst[16 * mt + g + 8] = o[mt][2] * f_a;
-      dst[kDecRedStride + 16 * mt + g + 8] = o[mt][3] * f_b;
+      dst[16 * mt + g] = o_sum[mt][0] * f_a;
+      dst[kDecRedStride + 16 * mt + g] = o_sum[mt][1] * f_b;
+      dst[16 * mt + g + 8] = o_sum[mt][2] * f_a;
+      dst[kDecRedStride + 16 * mt + g + 8] = o_sum[mt][3] * f_b;
     }
   }
   __syncthreads();
+  if constexpr (CLUSTER > 0) {
+    // ---- the splits of this (sequence, KV head) are one cluster: they read one another's partials in shared memory ----
+    const uint32_t mine = base + kDecClusterOffset;                // [G][132]: accumulator, maximum, sum
+    float* const own = reinterpret_cast<float*>(gen + kDecClusterOffset);
+    for (int i = tid; i < a.G * 128; i += kDecThreads) {
+      const int head = i >> 7, d = i & 127;
+      float sum = 0.f;
+#pragma unroll
+      for (int wi = 0; wi < kDecWarps; ++wi) sum += red[(wi * 8 + head) * kDecRedStride + d];
+      own[head * kDecPartFloats + d] = sum;
+    }
+    if (tid < a.G) {
+      float top = -INFINITY, l = 0.f;
+#pragma unroll
+      for (int wi = 0; wi < kDecWarps; ++wi) { top = fmaxf(top, wm[wi * 8 + tid]); l += wl[wi * 8 + tid]; }
+      own[tid * kDecPartFloats + 128] = top;
+      own[tid * kDecPartFloats + 129] = l;
+    }
+    cluster_sync();                                                // every split's partial is written ...
+    const int total = a.G * 128, lo = split * total / a.n_split, hi = (split + 1) * total / a.n_split;
+    for (int i = lo + tid; i < hi; i += kDecThreads) {             // each CTA forms its share of the output elements
+      const int head = i >> 7, d = i & 127;
+      float m[CLUSTER], l[CLUSTER], v[CLUSTER], top = -INFINITY;
+#pragma unroll
+      for (int s = 0; s < CLUSTER; ++s) {
+        if (s < a.n_split) {
+          const uint32_t at = cluster_addr(mine + head * kDecPartFloats * 4, s);
+          m[s] = ld_cluster_f32(at + 128 * 4);
+          l[s] = ld_cluster_f32(at + 129 * 4);
+          v[s] = ld_cluster_f32(at + d * 4);
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < CLUSTER; ++s) if (s < a.n_split) top = fmaxf(top, m[s]);
+      float sum[2] = {0.f, 0.f}, den[2] = {0.f, 0.f};
+#pragma unroll
+      for (int s = 0; s < CLUSTER; ++s) {
+        if (s < a.n_split) {
+          const float w = exp2f(m[s] - top);
+          den[s & 1] = fmaf(w, l[s], den[s & 1]);
+          sum[s & 1] = fmaf(w, v[s], sum[s & 1]);
+        }
+      }
+      a.out[((long long)(b * a.H_kv + h) * a.G + head) * 128 + d] = (sum[0] + sum[1]) / (den[0] + den[1]);
+    }
+    cluster_sync();                                                // ... and read, before a CTA of the cluster may leave
+    return;
+  }
   float* part = a.part + (((long long)(b * a.H_kv + h) * a.n_split + split) * a.G) * kDecPartFloats;
   for (int i = tid; i < a.G * 128; i += kDecThreads) {
     const int head = i >> 7, d = i & 127;
