@@ -763,7 +763,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
                   c.n_kv_heads, d.G, d.Wp, d.GWp, q_alloc, d.Lp,
                   reinterpret_cast<uint4*>(counts), ((long long)nseg * S_len + 3) / 4, ctrl + 1, fix_counts, nseg, ctrl,
                   c.lsh_tables, part * d.Wp, part * d.GWp, d.GW, part == 0 ? 1 : 0,
-                  (need_exact && !h->profiling) ? 1 : 0, ctrl + 8, (part == 0 && !h->profiling) ? 1 : 0};
+                  h->profiling ? 0 : 1, ctrl + 8, (part == 0 && !h->profiling) ? 1 : 0};
       dim3 grid(d.Lp / kQsigTables, c.n_kv_heads, c.batch);
       LKV_CUDA(launch_qsig(d.Kp, mapQ, h->mapPq, qa, grid, qsig_smem_bytes(q_alloc, d.Kp), st), "qsig_kernel");
       h->qsig_done_total += grid.x * grid.y * grid.z;
@@ -795,7 +795,8 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     a1.stat_rows = d.GWp;
     a1.stat_rows_alloc = ((d.GWp + 127) / 128) * 128;
     const uint32_t smem = stream_smem_bytes(kLse, a1.stat_rows_alloc, 0);
-    a1.overlap_prev = (need_lsh && !h->profiling) ? 1 : 0;      // beside the query-signature kernel
+    a1.overlap_prev = h->profiling ? 0 : 1;                       // beside the query-signature kernel, or, as the call's first
+    a1.wait_first = need_lsh ? 0 : 1;                             //   kernel, beside whatever is ahead in the stream
     a1.release_next = h->profiling ? 0 : 1;                       // the score pass starts as SMs fall free
     if (!h->profiling) {
       if (++h->lse_epoch == 0) h->lse_epoch = 1;
@@ -850,7 +851,8 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     a3.stat_rows_alloc = a3.stat_rows;
     a3.n_tiles = seg_tiles * d.n_chunks;
     const uint32_t smem = stream_smem_bytes(kProj, a3.stat_rows_alloc, d.TC * (2 << d.Kp));
-    a3.overlap_prev = (need_exact && !h->profiling) ? 1 : 0;     // beside the tail of the score pass
+    a3.overlap_prev = h->profiling ? 0 : 1;                       // beside the tail of the score pass
+    a3.wait_first = need_exact ? 0 : 1;                           //   or the query-signature kernel, whose results it needs first
     a3.release_next = h->profiling ? 0 : 1;                       // the selection waits for this pass's results
     a3.end_wait = a3.overlap_prev;                                // the selection kernel follows both
     const int grid = stream_grid(a3.n_tiles, h->num_sms);
