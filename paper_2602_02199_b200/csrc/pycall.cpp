@@ -23,15 +23,21 @@ decltype(&laser_kv_consensus_accumulate) f_consensus_accumulate;
 struct Args {
   PyObject* const* p;
   bool ok = true;
-  long long i64() {
-    const unsigned long long v = PyLong_AsUnsignedLongLongMask(*p++);
-    if (v == (unsigned long long)-1 && PyErr_Occurred()) ok = false;
-    return (long long)v;
+  long long integer(PyObject* o) {
+    if (!PyLong_Check(o)) {
+      if (ok) PyErr_Format(PyExc_TypeError, "int expected instead of %s", Py_TYPE(o)->tp_name);
+      ok = false;
+      return 0;
+    }
+    return (long long)PyLong_AsUnsignedLongLongMask(o);
   }
+  long long i64() { return integer(*p++); }
   int32_t i32() { return (int32_t)i64(); }
   void* ptr() { return reinterpret_cast<void*>(i64()); }
   float f32() {
-    const double v = PyFloat_AsDouble(*p++);
+    PyObject* o = *p++;
+    if (!ok) return 0.f;
+    const double v = PyFloat_AsDouble(o);
     if (v == -1.0 && PyErr_Occurred()) ok = false;
     return (float)v;
   }
@@ -43,11 +49,7 @@ struct Args {
       ok = false;
       return;
     }
-    for (int i = 0; i < N; ++i) {
-      const unsigned long long v = PyLong_AsUnsignedLongLongMask(PyTuple_GET_ITEM(t, i));
-      if (v == (unsigned long long)-1 && PyErr_Occurred()) ok = false;
-      s[i] = (int64_t)v;
-    }
+    for (int i = 0; i < N; ++i) s[i] = integer(PyTuple_GET_ITEM(t, i));
   }
 };
 

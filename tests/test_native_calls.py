@@ -1,5 +1,6 @@
 """The binding's native call path on the CPU: arguments reach the library as the library's own checks see them, and what is
 not a call is refused."""
+import numpy as np
 import pytest
 
 from paper_2602_02199_b200 import binding as Bn
@@ -47,6 +48,8 @@ def test_what_is_not_a_call_raises(native):
         native.two_stage_topk(0, 0)
     with pytest.raises(TypeError):
         native.two_stage_topk(0, 0, 1.5, 8, 1, 1, 1, 0, 0)
+    with pytest.raises(TypeError):
+        native.two_stage_topk(0, 0, np.int64(1), 8, 1, 1, 1, 0, 0)
     with pytest.raises(ValueError):
         native.decode_attention(0, 0, 16, (128,), 0.0, 16, 16, 64, 0)
     with pytest.raises(ValueError):
