@@ -157,16 +157,19 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
   grid_dependency_wait();
   allow_dependents();
 
-  // O^T, eight 16-dim row blocks: of the running tiles, and of those before. The MMAs' own accumulators do not round to nearest;
-  // added up outside them every few tiles, the result over 1636 entries is 1.4e-7 instead of 2.2e-7 from fp64, over 61,680
-  // 2.5e-7 instead of 1.3e-6. (Tile by tile a cache of 61,680 entries takes 1 % longer, short ones no longer.)
-  constexpr int kTilesPerSum = CLUSTER > 0 ? 1 : 4;
-  float o[8][4], o_sum[8][4];
+  // O^T, eight 16-dim row blocks. The MMAs' own accumulators do not round to nearest; splits of a cluster, which may be longer
+  // than the others, add them up outside tile by tile: 1.4e-7 instead of 2.2e-7 from fp64 over 1636 entries, in the same
+  // time. (By way of memory, where four layers of 61,680 entries took 0.6 % longer with it, o is the sum.)
+  constexpr bool kSumOutside = CLUSTER > 0;
+  float o[8][4], o_tiles[kSumOutside ? 8 : 1][4];
   float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;   // heads 2c and 2c+1
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) o[mt][i] = o_sum[mt][i] = 0.f;
+    for (int i = 0; i < 4; ++i) {
+      o[mt][i] = 0.f;
+      if constexpr (kSumOutside) o_tiles[mt][i] = 0.f;
+    }
 
   if (warp == kDecWarps) {
     // ---- producer: one lane keeps the ring full -----------------------------------------------------
@@ -250,8 +253,9 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
           l_a *= f_a; l_b *= f_b;
 #pragma unroll
           for (int mt = 0; mt < 8; ++mt) {
-            if (kTilesPerSum > 1) { o[mt][0] *= f_a; o[mt][1] *= f_b; o[mt][2] *= f_a; o[mt][3] *= f_b; }
-            o_sum[mt][0] *= f_a; o_sum[mt][1] *= f_b; o_sum[mt][2] *= f_a; o_sum[mt][3] *= f_b;
+            float* x = o[mt];
+            if constexpr (kSumOutside) x = o_tiles[mt];            // o is empty between tiles
+            x[0] *= f_a; x[1] *= f_b; x[2] *= f_a; x[3] *= f_b;
           }
         }
         const float p0 = exp2f(x0 - m_a), p1 = exp2f(x1 - m_b), p2 = exp2f(x2 - m_a), p3 = exp2f(x3 - m_b);
@@ -279,11 +283,11 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_empty(st));
-      if (kTilesPerSum == 1 || t % kTilesPerSum == kTilesPerSum - 1 || t == n_tiles - 1) {
+      if constexpr (kSumOutside) {
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) { o_sum[mt][i] += o[mt][i]; o[mt][i] = 0.f; }
+          for (int i = 0; i < 4; ++i) { o_tiles[mt][i] += o[mt][i]; o[mt][i] = 0.f; }
       }
     }
     // the warp's sums over its keys: lanes with equal c hold different keys
@@ -306,10 +310,12 @@ decode_split_kernel(const __grid_constant__ CUtensorMap map_k,    // cache K: (d
     float* dst = red + (warp * 8 + 2 * c) * kDecRedStride;
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) {
-      dst[16 * mt + g] = o_sum[mt][0] * f_a;
-      dst[kDecRedStride + 16 * mt + g] = o_sum[mt][1] * f_b;
-      dst[16 * mt + g + 8] = o_sum[mt][2] * f_a;
-      dst[kDecRedStride + 16 * mt + g + 8] = o_sum[mt][3] * f_b;
+      const float* x = o[mt];
+      if constexpr (kSumOutside) x = o_tiles[mt];
+      dst[16 * mt + g] = x[0] * f_a;
+      dst[kDecRedStride + 16 * mt + g] = x[1] * f_b;
+      dst[16 * mt + g + 8] = x[2] * f_a;
+      dst[kDecRedStride + 16 * mt + g + 8] = x[3] * f_b;
     }
   }
   __syncthreads();
