@@ -112,8 +112,9 @@ struct StreamArgs {
   uint32_t polls, poll_ns;     // budget of the hand-off waits: polls, and nanoseconds a poll may suspend
   int overlap_prev;    // launched (with the programmatic-serialization attribute) to start beside the kernel ahead
   int release_next;    // the kernel after this one was launched that way: let it take the SMs as they fall free
-  int wait_first;      // launched beside the kernel ahead, but nothing is read or written before that is complete: the launch and
-                       //   the set-up of barriers and tensor memory are hidden (80 segments of 1864 keys, exact only: 49.3 -> 46.3 us a call)
+  int wait_first;      // launched beside the kernel ahead, but nothing is read or written, and no tensor memory allocated, before that
+                       //   is complete: the launch and the set-up of the barriers are hidden (32 segments of 2048 keys, exact
+                       //   only, in a captured graph: 33.5 -> 31.4 us a call; 31.2 with the allocation ahead of the wait)
   int end_wait;        // wait for the grid ahead before this kernel ends, so that what follows in the stream follows both
   // Words in global memory that order kernels running beside each other without waiting for a whole
   // grid (which, besides coupling every CTA to the slowest one, takes microseconds after the grid's
@@ -867,12 +868,15 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
     fence_mbar_init();
     if (MODE == kProj) *reinterpret_cast<int*>(xch_s) = 0;      // items of the CTA's list of doubtful signs
   }
+  // Tensor memory is not held across a wait for another grid: a CTA of that grid on this SM may still have its own to
+  // allocate (the query-signature kernel releases this one before it does, and what a caller has ahead in the stream is
+  // not known here), and neither of the two would ever go on.
+  if (a.wait_first) grid_dependency_wait();
   if (warp == 1) { tmem_alloc(sm_tmem_slot, kTmemCols); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  if (a.wait_first) grid_dependency_wait();
   // (a score pass that itself started early releases its successor only once it has waited: see below)
   if (a.release_next) {
     if (a.gate_counter == nullptr) {
@@ -1034,8 +1038,7 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
       ok = (nmb == 2) ? lse_epilogue<64>(a, e, nmb) : lse_epilogue<32>(a, e, nmb);
     } else if constexpr (MODE == kScore) {
       // started beside the log-sum-exp pass: tiles are loaded and multiplied meanwhile; the normalisers
-      // of a segment are read once their flags are up (or, without flags, once that grid has completed)
-      if (a.overlap_prev && a.lse_flags == nullptr) grid_dependency_wait();
+      // of a segment are read once their flags are up
       // group g sums the query columns [c0, c1); widths are multiples of 16, at most 64
       const int cw = ((a.GW + kEpiGroups - 1) / kEpiGroups + 15) & ~15;
       const int c0 = e.wg * cw;
