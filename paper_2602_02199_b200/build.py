@@ -13,7 +13,7 @@ LIB = os.path.join(HERE, "liblaserkv.so")
 PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 API = os.path.join(HERE, "..", "include", "laser_kv.h")
 SOURCES = ["api.cu"]
-HEADERS = ["ptx.cuh", "theory_math.cuh", "stream_gemm.cuh", "aux_kernels.cuh", "query_proj.cuh", "decode_attn.cuh"]
+HEADERS = ["launch_rules.h", "ptx.cuh", "theory_math.cuh", "stream_gemm.cuh", "aux_kernels.cuh", "query_proj.cuh", "decode_attn.cuh"]
 
 
 def _nvcc() -> str:

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/laser_kv.h"
+#include "launch_rules.h"
 #include "aux_kernels.cuh"
 #include "stream_gemm.cuh"
 #include "query_proj.cuh"
@@ -433,21 +434,6 @@ laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st,
 }
 
 
-// Splits per (sequence, KV head) of a decode call: as many as fill the GPU's resident CTAs once, but at
-// most eight of up to 24 tiles and a third of the tiles above: a tile costs a CTA 0.3 us, a split's partials cost
-// the CTA that merges them about as much. us per layer in a captured graph, one tile per split against
-// three: 26 tiles x 8 heads 7.2 / 6.9, 52 x 8 9.2 / 8.2, 103 x 8 11.2 / 10.9, 52 x 4 heads of seven queries
-// 12.0 / 8.0; four tiles 5.0 / 5.3, hence the eight.
-int decode_splits(const laser_kv_ctx* h, long long len) {
-  const laser_kv_config_t& c = h->cfg;
-  long long n = (long long)h->num_sms * kDecCtasPerSm / ((long long)c.batch * c.n_kv_heads);
-  const long long tiles = (len + kDecTile - 1) / kDecTile;
-  const long long most = tiles <= 8 ? tiles : tiles <= 24 ? 8 : (tiles + 2) / 3;
-  if (n > most) n = most;
-  if (n > kDecMaxSplit) n = kDecMaxSplit;
-  return n < 1 ? 1 : (int)n;
-}
-
 // Slices of the projection pass of a select call. The SMs that held a query-signature CTA came 5 to 7 us later to the log-sum-exp
 // pass, and every SM goes from pass to pass as it is done, so the last CTAs of the projection pass start that much later and
 // the selection waited for them. They get fewer tiles, about 5 us less of them (eight of 160 columns), but not less than 55 %:
@@ -467,29 +453,6 @@ void weight_proj_slices(StreamArgs* a, int grid, int qsig_ctas, int abreast) {
   const long long w_less = less * a->w_early / per;
   const long long most = a->w_early * 45ll / 100;
   a->w_late = a->w_early - (int)(w_less < most ? w_less : most);
-}
-
-// Splits per (sequence, KV head) that merge inside a thread-block cluster (0: n_split of them by way of global memory, where
-// a partial goes to memory, is counted there and comes back to the CTA that merges). us per layer in a captured graph, by way of
-// memory against a cluster of at most eight: 8 heads of four queries and 4 tiles 5.2 / 3.5, 13 5.9 / 4.5, 26 7.2 / 6.3, 64 9.3 /
-// 8.5, 103 10.8 / 10.9; 4 heads of seven queries and 26 tiles 7.4 / 5.4. A cluster has to find room on one part of the GPU:
-// up to 256 CTAs in all do (264 of them 10.3 against 10.7, 280 14.3 against 10.8).
-// Longer caches of few heads with many queries: the general path's merge costs as much as its partials are large, a cluster
-// of sixteen reads the cache with fewer CTAs (4 heads of seven queries, 150 tiles 15.5 / 10.4, 512 24.5 / 21.2, 1024
-// 35.1 / 36.2; one head of eight, 512 28.4 / 18.5; 8 heads of four, 80 10.0 / 9.2, 255 16.9 / 16.6, 512 27.0 / 27.4; 4 heads
-// of two, 80 6.9 / 7.2). The inequality is where the two cross, from these and twenty more.
-int decode_cluster(const laser_kv_ctx* h, long long len, int n_split) {
-  const laser_kv_config_t& c = h->cfg;
-  const long long tiles = (len + kDecTile - 1) / kDecTile, heads = (long long)c.batch * c.n_kv_heads;
-  if (tiles <= 64) {
-    long long n = (long long)h->num_sms * kDecCtasPerSm / heads;
-    if (n > 8) n = 8;
-    if (n > tiles) n = tiles;
-    if (n <= 1) return 1;
-    return n * heads <= 256 ? (int)n : 0;
-  }
-  const long long G = c.n_q_heads / c.n_kv_heads;
-  return 16 * heads <= h->num_sms && 3 * (G * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
 }
 
 }  // namespace
@@ -1192,7 +1155,7 @@ laser_kv_status_t laser_kv_cache_view(laser_kv_handle_t h, int32_t layer, laser_
 size_t laser_kv_decode_attention_scratch_bytes(laser_kv_handle_t h) {
   if (!h) return 0;
   const laser_kv_config_t& c = h->cfg;
-  return (size_t)c.batch * c.n_q_heads * decode_splits(h, h->d.cap) * kDecPartFloats * sizeof(float);
+  return (size_t)c.batch * c.n_q_heads * decode_splits(h->num_sms, (long long)c.batch * c.n_kv_heads, h->d.cap) * kDecPartFloats * sizeof(float);
 }
 
 laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, const void* Q_dec,
@@ -1215,7 +1178,8 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   if (len < 1) return fail(h, LASER_KV_ERR_STATE, "decode_attention: layer %d cache is empty", layer);
   if (len > 0x7fffffffLL) return fail(h, LASER_KV_ERR_UNSUPPORTED, "decode_attention: cache longer than 2^31 entries");
   if (const laser_kv_status_t ds = check_device(h, "decode_attention")) return ds;
-  const int n_split = decode_splits(h, len);
+  const long long heads = (long long)c.batch * c.n_kv_heads;
+  const int n_split = decode_splits(h->num_sms, heads, len);
   const size_t need = (size_t)c.batch * c.n_q_heads * n_split * kDecPartFloats * sizeof(float);
   if (scratch_bytes < need) return fail(h, LASER_KV_ERR_CAPACITY, "decode_attention: scratch needs %zu bytes, got %zu", need, scratch_bytes);
 
@@ -1247,7 +1211,7 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   a.counters = reinterpret_cast<int*>(h->ws + h->carve.dec_count);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  const int n_cluster = decode_cluster(h, len, n_split);
+  const int n_cluster = decode_cluster(h->num_sms, heads, G, len, n_split);
   auto run = [&](auto kernel, std::atomic<unsigned long long>& limit_set, int n, bool any_cluster, int cluster) {
     a.n_split = n;
     const cudaError_t le = ensure_smem_limit(limit_set, kernel, (int)dec_smem_bytes(), any_cluster);

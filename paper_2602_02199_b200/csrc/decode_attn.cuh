@@ -33,21 +33,19 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "launch_rules.h"
 #include "ptx.cuh"
 #include "stream_gemm.cuh"
 
 namespace lkv {
 
-constexpr int kDecTile = 64;            // cache rows per stage
 constexpr int kDecBoxBytes = kDecTile * 128;   // one TMA box: 64 rows x 64 bf16
 constexpr int kDecStageBytes = 4 * kDecBoxBytes;   // K cols 0-63, K cols 64-127, V cols 0-63, V cols 64-127
 constexpr int kDecStages = 3;
 constexpr int kDecWarps = 4;            // consumer warps, 16 rows of every tile each
 constexpr int kDecThreads = (kDecWarps + 1) * 32;
-constexpr int kDecCtasPerSm = 2;
 constexpr int kDecMaxGroup = 8;         // query heads per KV head, at most (the N of the MMA)
 constexpr int kDecPartFloats = 128 + 4; // per (split, query head): accumulator, reference max, sum, padding to 16 bytes
-constexpr int kDecMaxSplit = 512;
 constexpr float kDecRescaleAt = 20.f;   // log2 units a score may exceed the reference maximum by
 constexpr uint32_t kDecClusterOffset = 20480;   // their partials in shared memory, behind the warps' merge buffer
 constexpr int kDecRedStride = 132;      // floats between heads in the merge buffer (bank spread)

@@ -1,0 +1,53 @@
+// How calls are cut into CTAs: rules on sizes alone, in plain C++ (tests/test_launch_rules.py compiles them for the host).
+#pragma once
+
+namespace lkv {
+
+constexpr int kDecTile = 64;            // cache rows per stage of the decode kernel
+constexpr int kDecCtasPerSm = 2;
+constexpr int kDecMaxSplit = 512;
+
+// Splits per (sequence, KV head) of a decode call whose partials go through memory: as many as fill the GPU's resident CTAs
+// once, but at most eight of up to 24 tiles and a third of the tiles above: a tile costs a CTA 0.3 us, a split's partials cost
+// the CTA that merges them about as much. us per layer in a captured graph, one tile per split against
+// three: 26 tiles x 8 heads 7.2 / 6.9, 52 x 8 9.2 / 8.2, 103 x 8 11.2 / 10.9, 52 x 4 heads of seven queries
+// 12.0 / 8.0; four tiles 5.0 / 5.3, hence the eight. `heads`: sequences x KV heads.
+inline int decode_splits(int num_sms, long long heads, long long len) {
+  long long n = (long long)num_sms * kDecCtasPerSm / heads;
+  const long long tiles = (len + kDecTile - 1) / kDecTile;
+  const long long most = tiles <= 8 ? tiles : tiles <= 24 ? 8 : (tiles + 2) / 3;
+  if (n > most) n = most;
+  if (n > kDecMaxSplit) n = kDecMaxSplit;
+  return n < 1 ? 1 : (int)n;
+}
+
+// Splits per (sequence, KV head) that merge inside a thread-block cluster (0: n_split of them by way of global memory, where
+// a partial goes to memory, is counted there and comes back to the CTA that merges). us per layer in a captured graph, by way of
+// memory against a cluster of at most eight: 8 heads of four queries and 4 tiles 5.2 / 3.5, 13 5.9 / 4.5, 26 7.2 / 6.3, 64 9.3 /
+// 8.5, 103 10.8 / 10.9; 4 heads of seven queries and 26 tiles 7.4 / 5.4. A cluster has to find room on one part of the GPU:
+// up to 256 CTAs in all do (264 of them 10.3 against 10.7, 280 14.3 against 10.8).
+// With few heads eight CTAs of more than six tiles each fall behind splits that have an SM each; a cluster of sixteen does not:
+// 4 heads of one query and 64 tiles 6.3 by way of memory / 7.0 eight / 6.4 sixteen, of four 6.7 / 7.2 / 6.5, 2 heads of two
+// and 50 tiles 6.4 / 6.6 / 6.2, 6 heads of eight and 64 0.79 / 0.72 of the time by way of memory. From 8 heads on clusters of
+// sixteen share SMs and are slower (8 heads of one, 50 tiles 6.5 / 6.7 / 7.2).
+// Longer caches of few heads with many queries: the general path's merge costs as much as its partials are large, a cluster
+// of sixteen reads the cache with fewer CTAs (one head of eight, 512 tiles 28.4 / 18.5; 4 heads of seven, 160 15.5 / 10.7, 512
+// 24.4 / 21.2, 1024 35.1 / 36.2; 8 heads of four, 80 8.3 / 8.5, 255 16.8 / 16.7, 512 27.0 / 27.4; 4 heads of two, 80 6.4 / 6.5).
+// The inequality is where the two cross for 1 to 9 heads and twelve lengths of 70 to 1024 tiles: at six queries and more to a
+// percent; for three to five the clusters it takes are up to 7 % slower at single lengths (5 heads of three, 320 tiles 14.9 /
+// 16.0; 4 of four, 100 7.3 / 7.7) and up to 13 % faster at others (6 of four, 80 8.1 / 7.0), and 2.1e-7 instead of 2.7e-7
+// to 4e-7 from fp64.
+inline int decode_cluster(int num_sms, long long heads, int group, long long len, int n_split) {
+  const long long tiles = (len + kDecTile - 1) / kDecTile;
+  if (tiles <= 64) {
+    if (tiles > 48 && heads <= 6 && 16 * heads <= num_sms) return 16;
+    long long n = (long long)num_sms * kDecCtasPerSm / heads;
+    if (n > 8) n = 8;
+    if (n > tiles) n = tiles;
+    if (n <= 1) return 1;
+    return n * heads <= 256 ? (int)n : 0;
+  }
+  return 16 * heads <= num_sms && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
+}
+
+}  // namespace lkv
