@@ -77,6 +77,7 @@ struct laser_kv_ctx {
   CUtensorMap mapPq;   // hyperplanes, box = the eight tables of one query-signature CTA
   EncodeTiledFn encode = nullptr;
   int num_sms = 1;
+  int cluster_room[kDecMaxCluster + 1] = {0};   // decode: clusters of each size that the device holds at once
   std::vector<long long> blocks_done;   // per layer: blocks processed
   std::vector<long long> entries_done;  // per layer: cache entries final per (sequence, KV head)
   std::vector<long long> tokens_done;   // per layer: tokens of the blocks processed
@@ -434,6 +435,33 @@ laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st,
 }
 
 
+template <int CLUSTER>
+cudaError_t decode_limits() {
+  static std::atomic<unsigned long long> limit_set{0};   // per instantiation
+  return ensure_smem_limit(limit_set, decode_split_kernel<CLUSTER>, (int)dec_smem_bytes(), CLUSTER > 8);
+}
+
+// How many clusters of `n` decode CTAs the current device holds at once; 0 also where it cannot say.
+template <int CLUSTER>
+int decode_cluster_room(int n) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n);
+  cfg.blockDim = dim3(kDecThreads);
+  cfg.dynamicSmemBytes = dec_smem_bytes();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = n;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int room = 0;
+  if (decode_limits<CLUSTER>() != cudaSuccess || cudaOccupancyMaxActiveClusters(&room, decode_split_kernel<CLUSTER>, &cfg) != cudaSuccess) {
+    cudaGetLastError();       // not an error of the call: the splits merge by way of memory
+    return 0;
+  }
+  return room;
+}
+
 // Slices of the projection pass of a select call. The SMs that held a query-signature CTA came 5 to 7 us later to the log-sum-exp
 // pass, and every SM goes from pass to pass as it is done, so the last CTAs of the projection pass start that much later and
 // the selection waited for them. They get fewer tiles, about 5 us less of them (eight of 160 columns), but not less than 55 %:
@@ -537,6 +565,8 @@ laser_kv_status_t laser_kv_init(const laser_kv_config_t* cfg, const void* hyperp
   h->ws = static_cast<uint8_t*>(workspace);
   h->encode = reinterpret_cast<EncodeTiledFn>(fn);
   h->num_sms = prop.multiProcessorCount;
+  for (int n = 2; n <= 8; ++n) h->cluster_room[n] = decode_cluster_room<8>(n);
+  h->cluster_room[16] = decode_cluster_room<16>(16);
   const size_t per = (size_t)cfg->n_layers * cfg->batch * cfg->n_kv_heads * (size_t)d.cap;
   uint8_t* cm = static_cast<uint8_t*>(cache_mem);
   h->cacheK = reinterpret_cast<uint16_t*>(cm);
@@ -1211,18 +1241,16 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   a.counters = reinterpret_cast<int*>(h->ws + h->carve.dec_count);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  const int n_cluster = decode_cluster(h->num_sms, heads, G, len, n_split);
-  auto run = [&](auto kernel, std::atomic<unsigned long long>& limit_set, int n, bool any_cluster, int cluster) {
+  const int n_cluster = decode_cluster(h->num_sms, heads, G, len, n_split, h->cluster_room);
+  auto run = [&](auto kernel, cudaError_t limits, int n, int cluster) {
+    if (limits != cudaSuccess) return limits;
     a.n_split = n;
-    const cudaError_t le = ensure_smem_limit(limit_set, kernel, (int)dec_smem_bytes(), any_cluster);
-    if (le != cudaSuccess) return le;
     return launch_clusters(kernel, dim3((unsigned)n, (unsigned)c.n_kv_heads, (unsigned)c.batch), kDecThreads, dec_smem_bytes(), st, true,
                            cluster, maps.k, maps.v, a);
   };
-  static std::atomic<unsigned long long> limit0{0}, limit8{0}, limit16{0};
-  if (n_cluster == 0) e = run(decode_split_kernel<0>, limit0, n_split, false, 1);
-  else if (n_cluster <= 8) e = run(decode_split_kernel<8>, limit8, n_cluster, false, n_cluster);
-  else e = run(decode_split_kernel<16>, limit16, n_cluster, true, n_cluster);
+  if (n_cluster == 0) e = run(decode_split_kernel<0>, decode_limits<0>(), n_split, 1);
+  else if (n_cluster <= 8) e = run(decode_split_kernel<8>, decode_limits<8>(), n_cluster, n_cluster);
+  else e = run(decode_split_kernel<16>, decode_limits<16>(), n_cluster, n_cluster);
   if (e != cudaSuccess) return fail(h, LASER_KV_ERR_CUDA, "decode_split_kernel launch: %s", cudaGetErrorString(e));
   return LASER_KV_OK;
 }

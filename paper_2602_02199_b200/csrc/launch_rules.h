@@ -6,12 +6,14 @@ namespace lkv {
 constexpr int kDecTile = 64;            // cache rows per stage of the decode kernel
 constexpr int kDecCtasPerSm = 2;
 constexpr int kDecMaxSplit = 512;
+constexpr int kDecMaxCluster = 16;
 
 // Splits per (sequence, KV head) of a decode call whose partials go through memory: as many as fill the GPU's resident CTAs
 // once, but at most eight of up to 24 tiles and a third of the tiles above: a tile costs a CTA 0.3 us, a split's partials cost
 // the CTA that merges them about as much. us per layer in a captured graph, one tile per split against
 // three: 26 tiles x 8 heads 7.2 / 6.9, 52 x 8 9.2 / 8.2, 103 x 8 11.2 / 10.9, 52 x 4 heads of seven queries
-// 12.0 / 8.0; four tiles 5.0 / 5.3, hence the eight. `heads`: sequences x KV heads.
+// 12.0 / 8.0; four tiles 5.0 / 5.3, hence the eight (short caches come here where clusters do not fit, see below). `heads`:
+// sequences x KV heads.
 inline int decode_splits(int num_sms, long long heads, long long len) {
   long long n = (long long)num_sms * kDecCtasPerSm / heads;
   const long long tiles = (len + kDecTile - 1) / kDecTile;
@@ -37,17 +39,21 @@ inline int decode_splits(int num_sms, long long heads, long long len) {
 // percent; for three to five the clusters it takes are up to 7 % slower at single lengths (5 heads of three, 320 tiles 14.9 /
 // 16.0; 4 of four, 100 7.3 / 7.7) and up to 13 % faster at others (6 of four, 80 8.1 / 7.0), and 2.1e-7 instead of 2.7e-7
 // to 4e-7 from fp64.
-inline int decode_cluster(int num_sms, long long heads, int group, long long len, int n_split) {
+// `room`: how many clusters of each size (up to kDecMaxCluster) the device holds at once. Only sizes of which it holds
+// all the call's are used; a device, or a part of one, that holds none of a size would refuse the launch. The B200's
+// 148 SMs hold 33 of eight, 14 of sixteen.
+inline int decode_cluster(int num_sms, long long heads, int group, long long len, int n_split, const int* room) {
   const long long tiles = (len + kDecTile - 1) / kDecTile;
+  const bool sixteen = 16 * heads <= num_sms && heads <= room[16];
   if (tiles <= 64) {
-    if (tiles > 48 && heads <= 6 && 16 * heads <= num_sms) return 16;
+    if (tiles > 48 && heads <= 6 && sixteen) return 16;
     long long n = (long long)num_sms * kDecCtasPerSm / heads;
     if (n > 8) n = 8;
     if (n > tiles) n = tiles;
     if (n <= 1) return 1;
-    return n * heads <= 256 ? (int)n : 0;
+    return n * heads <= 256 && heads <= room[n] ? (int)n : 0;
   }
-  return 16 * heads <= num_sms && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
+  return sixteen && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
 }
 
 }  // namespace lkv

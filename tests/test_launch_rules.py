@@ -8,11 +8,13 @@ import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_02199_b200", "csrc")
 SMS = 148
+# clusters of 0 to 16 decode CTAs that such a device holds at once (9 to 15 are not used)
+ROOM = [0, 0, 148, 93, 71, 56, 45, 37, 33, 0, 0, 0, 0, 0, 0, 0, 14]
 SHIM = """
 #include "launch_rules.h"
 extern "C" int decode_splits(int sms, long long heads, long long len) { return lkv::decode_splits(sms, heads, len); }
-extern "C" int decode_cluster(int sms, long long heads, int group, long long len) {
-  return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len));
+extern "C" int decode_cluster(int sms, long long heads, int group, long long len, const int* room) {
+  return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len), room);
 }
 """
 
@@ -29,11 +31,15 @@ def rules(tmp_path_factory):
     return C.CDLL(lib)
 
 
+def cluster(rules, heads, group, length, room=ROOM):
+    return rules.decode_cluster(SMS, C.c_longlong(heads), group, C.c_longlong(length), (C.c_int * 17)(*room))
+
+
 def test_decode_splits_are_whole_tiles_and_never_empty(rules):
     for heads in (1, 3, 8, 33, 64, 400):
         for tiles in list(range(1, 200)) + [964, 4000]:
             n = rules.decode_splits(SMS, C.c_longlong(heads), C.c_longlong(64 * tiles))
-            c = rules.decode_cluster(SMS, C.c_longlong(heads), 4, C.c_longlong(64 * tiles - 63))
+            c = cluster(rules, heads, 4, 64 * tiles - 63)
             assert 1 <= n <= min(tiles, 512) and 0 <= c <= min(tiles, 16)
 
 
@@ -42,4 +48,17 @@ def test_few_heads_give_no_cta_more_than_six_tiles_of_a_short_cache(rules, heads
     # seven and eight tiles a CTA cost up to 12 % against splits by way of memory that have an SM each
     for group in range(1, 9):
         for tiles in range(1, 65):
-            assert -(-tiles // rules.decode_cluster(SMS, C.c_longlong(heads), group, C.c_longlong(64 * tiles))) <= 6
+            assert -(-tiles // cluster(rules, heads, group, 64 * tiles)) <= 6
+
+
+@pytest.mark.parametrize("room", [[0] * 17, [0, 0] + [1] * 7 + [0] * 8, ROOM[:9] + [0] * 8, [n // 4 for n in ROOM]])
+def test_clusters_the_device_does_not_hold_are_not_launched(rules, room):
+    fewer = 0
+    for heads in (1, 2, 4, 6, 8, 9, 16, 32, 40, 64, 128, 300):
+        for group in (1, 4, 8):
+            for tiles in (1, 2, 7, 8, 26, 48, 49, 64, 65, 100, 255, 964):
+                n, usual = cluster(rules, heads, group, 64 * tiles, room), cluster(rules, heads, group, 64 * tiles)
+                assert n <= 1 or heads <= room[n]
+                assert n == usual or heads > room[usual]       # what fits is launched as ever
+                fewer += n != usual
+    assert fewer > 0
