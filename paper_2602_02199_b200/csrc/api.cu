@@ -462,27 +462,6 @@ int decode_cluster_room(int n) {
   return room;
 }
 
-// Slices of the projection pass of a select call. The SMs that held a query-signature CTA came 5 to 7 us later to the log-sum-exp
-// pass, and every SM goes from pass to pass as it is done, so the last CTAs of the projection pass start that much later and
-// the selection waited for them. They get fewer tiles, about 5 us less of them (eight of 160 columns), but not less than 55 %:
-// sixteen calls of one block of 8192 tokens 978 -> 953 us (at least 50 %: 959, 60 %: 961, 70 %: 969), 64k in one call
-// 203 -> 198, 32k 101.8 -> 98.8.
-// Where the keys outgrow the L2 cache (above 64 MB), CTAs with the same keys and different chunks must stay together, or the
-// keys come from memory again for each chunk: unequal slices one behind the other took a 128k layer from 399 to 432 us in a
-// burst, slices abreast leave it as it was (four sequences of 128k tokens 622 -> 614 us, 64k 179 -> 176). With keys in the
-// cache the slices one behind the other are the better ones by 1 %.
-constexpr long long kProjAbreastBytes = 64ll << 20;
-void weight_proj_slices(StreamArgs* a, int grid, int qsig_ctas, int abreast) {
-  if (qsig_ctas >= grid || grid % abreast) return;
-  const long long per = 1000 * a->n_tiles / grid, less = 1000ll * 8 * 160 / a->stat_rows;      // thousandths of a tile
-  a->abreast = abreast;
-  a->n_late = qsig_ctas;
-  a->w_early = (int)(per < 1000000 ? per : 1000000);
-  const long long w_less = less * a->w_early / per;
-  const long long most = a->w_early * 45ll / 100;
-  a->w_late = a->w_early - (int)(w_less < most ? w_less : most);
-}
-
 }  // namespace
 
 extern "C" {
@@ -850,7 +829,8 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     a3.end_wait = a3.overlap_prev;                                // the selection kernel follows both
     const int grid = stream_grid(a3.n_tiles, h->num_sms);
     if (need_exact && !h->profiling)
-      weight_proj_slices(&a3, grid, d.Lp / kQsigTables * c.n_kv_heads * c.batch, seg_tiles * kTileBytes > kProjAbreastBytes ? d.n_chunks : 1);
+      a3.slices = proj_slices(h->num_sms, grid, a3.n_tiles, a3.stat_rows, base_ctas, (long long)d.Lp / kQsigTables * c.n_kv_heads * c.batch,
+                              seg_tiles * kTileBytes > kProjAbreastBytes ? d.n_chunks : 1);
     a3.fix_list = fix_list_items(d.fix_cap, (size_t)d.nseg_max, grid);
     LKV_CUDA(launch_proj(d.Kp, d.TC, mapK, h->mapP, a3, grid, smem, st),
              "projection pass");

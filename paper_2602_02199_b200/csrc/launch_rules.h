@@ -1,6 +1,12 @@
 // How calls are cut into CTAs: rules on sizes alone, in plain C++ (tests/test_launch_rules.py compiles them for the host).
 #pragma once
 
+#ifdef __CUDACC__
+#define LKV_HOST_DEVICE __host__ __device__
+#else
+#define LKV_HOST_DEVICE
+#endif
+
 namespace lkv {
 
 constexpr int kDecTile = 64;            // cache rows per stage of the decode kernel
@@ -54,6 +60,46 @@ inline int decode_cluster(int num_sms, long long heads, int group, long long len
     return n * heads <= 256 && heads <= room[n] ? (int)n : 0;
   }
   return sixteen && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
+}
+
+// Slices of the projection pass of a select call. The SMs that held a query-signature CTA come 5 to 7 us later to the log-sum-exp
+// pass, and every SM goes from pass to pass as it is done, so the last CTAs of the projection pass start that much later and
+// the selection waited for them. They get fewer tiles, about 5 us less of them (eight of 160 columns), but not less than 55 %:
+// sixteen calls of one block of 8192 tokens 978 -> 953 us (at least 50 %: 959, 60 %: 961, 70 %: 969), 64k in one call
+// 203 -> 198, 32k 101.8 -> 98.8.
+// Where the keys outgrow the L2 cache (above 64 MB), CTAs with the same keys and different chunks must stay together, or the
+// keys come from memory again for each chunk: unequal slices one behind the other took a 128k layer from 399 to 432 us in a
+// burst, slices abreast leave it as it was (four sequences of 128k tokens 622 -> 614 us, 64k 179 -> 176). With keys in the
+// cache the slices one behind the other are the better ones by 1 %.
+constexpr long long kProjAbreastBytes = 64ll << 20;
+struct ProjSlices {
+  int n_late, w_late, w_early;   // the last n_late CTAs' slices are to the others' as w_late to w_early; all 0: equal slices
+  int abreast;                   // > 1: the sequence is cut into that many equal parts, CTAs c, c + 1, ... at the same place of each
+};
+
+// `grid` CTAs over n_tiles tiles of stat_rows columns, behind a log-sum-exp pass of lse_ctas CTAs that started beside qsig_ctas of the
+// query-signature kernel. Late are only the log-sum-exp CTAs that found no SM free: with few tiles in all, weights for every SM
+// with a signature CTA gave some CTAs a second tile for nothing (64 tiles of one head 34.1 us a call with equal slices, 34.9 so
+// weighted; 128 tiles of 16 segments 25.3 / 26.5, of 2 heads 28.4 / 29.9).
+inline ProjSlices proj_slices(int num_sms, int grid, long long n_tiles, int stat_rows, int lse_ctas, long long qsig_ctas, int abreast) {
+  long long late = lse_ctas + qsig_ctas - num_sms;
+  if (late > qsig_ctas) late = qsig_ctas;
+  if (late <= 0 || late >= grid || grid % abreast) return ProjSlices{0, 0, 0, 0};
+  const long long per = 1000 * n_tiles / grid, less = 1000ll * 8 * 160 / stat_rows;      // thousandths of a tile
+  ProjSlices s;
+  s.abreast = abreast;
+  s.n_late = (int)late;
+  s.w_early = (int)(per < 1000000 ? per : 1000000);
+  const long long w_less = less * s.w_early / per, most = s.w_early * 45ll / 100;
+  s.w_late = s.w_early - (int)(w_less < most ? w_less : most);
+  return s;
+}
+
+// First tile of the c-th of n slices of `part` tiles, of which the last are those of the CTAs that start late.
+LKV_HOST_DEVICE inline long long weighted_begin(long long part, int c, int n, const ProjSlices& s) {
+  const int early = n - (s.n_late + s.abreast - 1) / s.abreast;
+  const long long w = (long long)(c < early ? c : early) * s.w_early + (long long)(c > early ? c - early : 0) * s.w_late;
+  return part * w / ((long long)early * s.w_early + (long long)(n - early) * s.w_late);
 }
 
 }  // namespace lkv

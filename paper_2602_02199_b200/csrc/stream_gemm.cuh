@@ -32,6 +32,7 @@
 // All cross-warp hand-offs are mbarriers with bounded waits; there is no CTA-wide barrier
 // inside the tile loop.
 #pragma once
+#include "launch_rules.h"
 #include "ptx.cuh"
 #include "theory_math.cuh"
 
@@ -83,10 +84,7 @@ struct StreamArgs {
   long long n_tiles;   // tiles of this launch: nseg * tiles_in_block (* n_chunks for kProj)
   int lse_ctas;        // grid of the kLse launch over the same segments (slot arithmetic)
   int n_slot;          // log-sum-exp partial slots per segment
-  // kProj: the last n_late CTAs of the grid start late, on SMs that held a CTA of the query-signature kernel, and take slices
-  // that are to the others' as w_late to w_early (both 0: all slices are equal and follow one another). With `abreast`
-  // > 1 the sequence is cut into that many equal parts and CTAs c, c + 1, ... work abreast at the same place of each.
-  int n_late, w_late, w_early, abreast;
+  ProjSlices slices;   // kProj: unequal slices for the CTAs that start late, on SMs that held a CTA of the query-signature kernel
   int stat_rows;       // rows of the stationary operand (GW, or tables_per_chunk * lsh_bits)
   int stat_rows_alloc; // rows reserved per 64-column half in shared memory (multiple of 8)
   int n_chunks, tables_per_chunk, lsh_bits, lsh_tables;
@@ -132,13 +130,6 @@ __device__ __forceinline__ void record_status(int* status, int code) {
 // The CTA whose slice [c*T/G, (c+1)*T/G) of a T-tile sequence split over G CTAs holds tile x.
 __host__ __device__ inline int cta_of_tile(long long x, long long T, int G) {
   return (int)(((x + 1) * G - 1) / T);
-}
-
-// First tile of the c-th of n slices of `part` tiles, of which the last are those of the CTAs that start late.
-__device__ __forceinline__ long long weighted_begin(long long part, int c, int n, const StreamArgs& a) {
-  const int early = n - (a.n_late + a.abreast - 1) / a.abreast;
-  const long long w = (long long)min(c, early) * a.w_early + (long long)max(0, c - early) * a.w_late;
-  return part * w / ((long long)early * a.w_early + (long long)(n - early) * a.w_late);
 }
 
 // Position in the tile sequence: hyperplane chunk, (sequence, KV head) pair, block, tile in block.
@@ -807,11 +798,11 @@ stream_kernel(const __grid_constant__ CUtensorMap map_keys,   // K: (d, token, h
 
   // ---- this CTA's slice of the tile sequence ------------------------------------------------
   long long x_begin, x_end;
-  if (MODE == kProj && a.w_early > 0) {
-    const int n = gridDim.x / a.abreast, c = blockIdx.x / a.abreast;
-    const long long part = a.n_tiles / a.abreast, first = part * (blockIdx.x % a.abreast);
-    x_begin = first + weighted_begin(part, c, n, a);
-    x_end = first + weighted_begin(part, c + 1, n, a);
+  if (MODE == kProj && a.slices.w_early > 0) {
+    const int abreast = a.slices.abreast, n = gridDim.x / abreast, c = blockIdx.x / abreast;
+    const long long part = a.n_tiles / abreast, first = part * (blockIdx.x % abreast);
+    x_begin = first + weighted_begin(part, c, n, a.slices);
+    x_end = first + weighted_begin(part, c + 1, n, a.slices);
   } else {
     x_begin = (long long)blockIdx.x * a.n_tiles / gridDim.x;
     x_end = (long long)(blockIdx.x + 1) * a.n_tiles / gridDim.x;

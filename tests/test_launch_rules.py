@@ -16,6 +16,16 @@ extern "C" int decode_splits(int sms, long long heads, long long len) { return l
 extern "C" int decode_cluster(int sms, long long heads, int group, long long len, const int* room) {
   return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len), room);
 }
+extern "C" int proj_slices(int sms, int grid, long long tiles, int rows, int lse, long long qsig, int abreast, int* begin) {
+  const lkv::ProjSlices s = lkv::proj_slices(sms, grid, tiles, rows, lse, qsig, abreast);
+  for (int c = 0; s.w_early > 0 && c < grid; ++c) {       // as the kernel: begin and end of every CTA's slice
+    const int n = grid / s.abreast;
+    const long long part = tiles / s.abreast, first = part * (c % s.abreast);
+    begin[2 * c] = (int)(first + lkv::weighted_begin(part, c / s.abreast, n, s));
+    begin[2 * c + 1] = (int)(first + lkv::weighted_begin(part, c / s.abreast + 1, n, s));
+  }
+  return s.n_late;
+}
 """
 
 
@@ -62,3 +72,36 @@ def test_clusters_the_device_does_not_hold_are_not_launched(rules, room):
                 assert n == usual or heads > room[usual]       # what fits is launched as ever
                 fewer += n != usual
     assert fewer > 0
+
+
+def slices(rules, seg_tiles, chunks, rows, qsig, abreast):
+    """(CTAs that start late, [begin, end) of every CTA's slice or None where they are equal)."""
+    lse, grid = min(SMS, seg_tiles), min(SMS, seg_tiles * chunks)
+    out = (C.c_int * (2 * grid))()
+    late = rules.proj_slices(SMS, grid, C.c_longlong(seg_tiles * chunks), rows, lse, C.c_longlong(qsig), abreast, out)
+    return late, list(zip(out[::2], out[1::2])) if late else None
+
+
+@pytest.mark.parametrize("rows", [64, 128, 160, 192])
+def test_slices_of_the_projection_pass_are_the_tiles_in_turn(rules, rows):
+    weighted = 0
+    for seg_tiles in list(range(1, 300, 7)) + [1024, 8192, 65536, 300000]:
+        for chunks in (1, 2, 3, 4, 5, 8):
+            for qsig in (1, 4, 16, 64, 147, 148, 500):
+                for abreast in {1, chunks}:
+                    late, cut = slices(rules, seg_tiles, chunks, rows, qsig, abreast)
+                    if cut is None:
+                        continue
+                    weighted += 1
+                    assert 0 < late <= qsig and all(b <= e for b, e in cut)
+                    ends = sorted(x for x in cut if x[0] < x[1])
+                    assert ends[0][0] == 0 and ends[-1][1] == seg_tiles * chunks
+                    assert all(a[1] == b[0] for a, b in zip(ends, ends[1:]))
+    assert weighted > 100
+
+
+@pytest.mark.parametrize("seg_tiles,chunks,qsig", [(48, 1, 4), (64, 1, 16), (64, 2, 4), (84, 4, 64), (96, 1, 16), (128, 1, 16), (132, 1, 16)])
+def test_slices_are_equal_where_no_cta_starts_late(rules, seg_tiles, chunks, qsig):
+    # every log-sum-exp CTA finds an SM without a signature CTA: a slice of two tiles beside one of none would take a tile longer
+    assert slices(rules, seg_tiles, chunks, 160, qsig, 1) == (0, None)
+    assert slices(rules, SMS - qsig + 1, chunks, 160, qsig, 1)[0] == 1
