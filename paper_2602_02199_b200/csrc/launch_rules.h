@@ -62,6 +62,10 @@ inline int decode_cluster(int num_sms, long long heads, int group, long long len
   return sixteen && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
 }
 
+// Score pass: log-sum-exp partials of a column that a warp fetches at a time. A segment with more is shared by a group's four warps.
+constexpr int kLseBatch = 5;
+LKV_HOST_DEVICE inline bool lse_split(int partials) { return partials > kLseBatch; }
+
 // Slices of the projection pass of a select call. The SMs that held a query-signature CTA come 5 to 7 us later to the log-sum-exp
 // pass, and every SM goes from pass to pass as it is done, so the last CTAs of the projection pass start that much later and
 // the selection waited for them. They get fewer tiles, about 5 us less of them (eight of 160 columns), but not less than 55 %:

@@ -60,8 +60,6 @@ __host__ __device__ constexpr int proj_acc_stride(int kbits, int tc) { return (k
 __host__ __device__ constexpr int proj_num_acc(int kbits, int tc) {
   return 512 / proj_acc_stride(kbits, tc) < kMaxAcc ? 512 / proj_acc_stride(kbits, tc) : kMaxAcc;
 }
-constexpr int kLseSplitAt = 8;                // partials of a segment above which the group's warps share the fetching
-constexpr int kLseBatch = 5;                  // log-sum-exp partials of a column fetched at a time
 constexpr int kMaxStreamCtas = 256;            // upper bound of the persistent grid (slot arithmetic)
 constexpr int kPolyPairsOf32 = 10;             // of every 32 column pairs, this many take 2^x on the FMA pipe
 
@@ -500,6 +498,92 @@ __device__ __forceinline__ bool lse_epilogue(const StreamArgs& a, const EpiCtx& 
   return true;
 }
 
+// Minus the log2-sum-exp2 of a warp's NC query columns over segment `seg`, into the warp's `lw`, from the partials of the CTAs
+// that covered the segment. One partial is a round trip to L2 of about 0.7 us, after another one for its flag. Up to kLseBatch
+// partials are fetched by every warp, all at once. More (few segments in the call, each shared by many CTAs) are split over the
+// group's four warps, which exchange their parts through shared memory: 19 partials, sixteen calls of one block of 8192 tokens,
+// 958 -> 921 us, calls of two blocks of 4096 276 -> 268; six or seven, 24 segments of 2048 keys with 192 queries a head, 42.2 us by
+// every warp in two batches, 41.3 split. Batches of eight do as well there, but not where 4 to 5 partials are fetched (64 segments of
+// 4096 keys 95.0 -> 96.1). In a function of its own this costs the loop over the tiles no registers (30.1 -> 29.4 us of it there).
+template <int NC>
+__device__ __forceinline__ bool score_normalisers(const StreamArgs& a, const EpiCtx& e, int c0, float* lw, int seg, int tib, uint32_t& exchanges) {
+  const long long first = (long long)seg * a.tiles_in_block;
+  const int cf = cta_of_tile(first, a.n_tiles, a.lse_ctas);
+  const int n_used = cta_of_tile(first + a.tiles_in_block - 1, a.n_tiles, a.lse_ctas) - cf + 1;
+  const bool split = lse_split(n_used);
+  const int first_slot = split ? e.quarter : 0, step = split ? 4 : 1;
+  bool ready = true;
+  if (a.lse_flags) {
+    // the log-sum-exp pass may still be running: wait for the flags of the partials this warp fetches
+    for (int s2 = first_slot + step * e.lane; s2 < n_used && ready; s2 += 32 * step)   // few long segments: more CTAs per segment than lanes
+      ready = wait_flag_equals(a.lse_flags + (size_t)seg * a.n_slot + s2, a.lse_epoch,
+                               a.poll_ns == 0 ? a.polls : kMaxFlagPolls);
+    if (!__all_sync(0xffffffffu, ready)) return false;
+  }
+  __syncwarp();
+  constexpr int NH = (NC + 31) / 32;
+  float mx[NH], sum[NH];
+#pragma unroll
+  for (int half = 0; half < NH; ++half) { mx[half] = -INFINITY; sum[half] = 0.f; }
+  const float2* p = a.lse_part + (size_t)seg * a.n_slot * a.GW + c0 + e.lane;
+  for (int s0 = first_slot; s0 < n_used; s0 += step * kLseBatch) {
+    float2 pe[NH][kLseBatch];
+#pragma unroll
+    for (int i = 0; i < kLseBatch; ++i)
+#pragma unroll
+      for (int half = 0; half < NH; ++half)
+        pe[half][i] = (s0 + step * i < n_used && e.lane + 32 * half < NC) ? __ldcg(p + (size_t)(s0 + step * i) * a.GW + 32 * half)
+                                                                          : make_float2(-INFINITY, 0.f);
+#pragma unroll
+    for (int half = 0; half < NH; ++half) {
+      float m2 = mx[half];
+#pragma unroll
+      for (int i = 0; i < kLseBatch; ++i) m2 = fmaxf(m2, pe[half][i].x);
+      if (m2 == -INFINITY) continue;
+      if (s0 > first_slot) sum[half] *= exp2f(mx[half] - m2);
+#pragma unroll
+      for (int i = 0; i < kLseBatch; ++i)
+        if (pe[half][i].x != -INFINITY) sum[half] += pe[half][i].y * exp2f(pe[half][i].x - m2);
+      mx[half] = m2;
+    }
+  }
+  if (split) {
+    float2* ex = reinterpret_cast<float2*>(e.xch_s + kXchBytes) + e.wg * 4 * kEpiCols;     // [4 groups][4 warps][64 columns]
+    const uint32_t bar_put = e.bar_norm + 16 * e.wg, bar_got = bar_put + 8;
+    if (!mbar_wait(bar_got, (exchanges + 1) & 1, a.polls, a.poll_ns)) return false;        // passes for the first
+#pragma unroll
+    for (int half = 0; half < NH; ++half) ex[e.quarter * kEpiCols + e.lane + 32 * half] = make_float2(mx[half], sum[half]);
+    __syncwarp();
+    if (e.lane == 0) mbar_arrive(bar_put);
+    if (!mbar_wait(bar_put, exchanges & 1, a.polls, a.poll_ns)) return false;
+#pragma unroll
+    for (int half = 0; half < NH; ++half) {
+      float2 pe[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) pe[i] = ex[i * kEpiCols + e.lane + 32 * half];
+      mx[half] = fmaxf(fmaxf(pe[0].x, pe[1].x), fmaxf(pe[2].x, pe[3].x));
+      sum[half] = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (pe[i].x != -INFINITY) sum[half] += pe[i].y * exp2f(pe[i].x - mx[half]);
+    }
+    __syncwarp();
+    if (e.lane == 0) mbar_arrive(bar_got);
+    ++exchanges;
+  }
+#pragma unroll
+  for (int half = 0; half < NH; ++half) {
+    const int j = e.lane + 32 * half;
+    if (j < NC) {
+      const float lse = mx[half] + log2f(sum[half]);
+      if (tib == 0 && e.quarter == 0) a.lse2[(size_t)seg * a.lse2_stride + a.lse2_off + c0 + j] = lse;
+      lw[j] = -lse;
+    }
+  }
+  __syncwarp();
+  return true;
+}
+
 // kScore: NC query columns [c0, c0 + NC) per thread; the groups' sums meet in group 0.
 template <int NC>
 __device__ __forceinline__ bool score_epilogue(const StreamArgs& a, const EpiCtx& e, int c0) {
@@ -515,85 +599,7 @@ __device__ __forceinline__ bool score_epilogue(const StreamArgs& a, const EpiCtx
     int n = min(left, a.tiles_in_block - tib);
     left -= n;
     if constexpr (NC > 0) {
-      // log2-sum-exp2 of this warp's queries from the partials of the CTAs that covered the segment
-      const long long first = (long long)seg * a.tiles_in_block;
-      const int cf = cta_of_tile(first, a.n_tiles, a.lse_ctas);
-      const int n_used = cta_of_tile(first + a.tiles_in_block - 1, a.n_tiles, a.lse_ctas) - cf + 1;
-      // One partial is a round trip to L2 of about 0.7 us, after another one for its flag. Up to kLseSplitAt partials are
-      // fetched by every warp, kLseBatch at a time. More (few segments in the call, each shared by many CTAs) are split over
-      // the group's four warps, which exchange their parts through shared memory: 19 partials, sixteen calls of one block of
-      // 8192 tokens, 958 -> 921 us, calls of two blocks of 4096 276 -> 268.
-      const bool split = n_used > kLseSplitAt;
-      const int first_slot = split ? e.quarter : 0, step = split ? 4 : 1;
-      bool ready = true;
-      if (a.lse_flags) {
-        // the log-sum-exp pass may still be running: wait for the flags of the partials this warp fetches
-        for (int s2 = first_slot + step * e.lane; s2 < n_used && ready; s2 += 32 * step)   // few long segments: more CTAs per segment than lanes
-          ready = wait_flag_equals(a.lse_flags + (size_t)seg * a.n_slot + s2, a.lse_epoch,
-                                   a.poll_ns == 0 ? a.polls : kMaxFlagPolls);
-        if (!__all_sync(0xffffffffu, ready)) return false;
-      }
-      __syncwarp();
-      constexpr int NH = (NC + 31) / 32;
-      float mx[NH], sum[NH];
-#pragma unroll
-      for (int half = 0; half < NH; ++half) { mx[half] = -INFINITY; sum[half] = 0.f; }
-      const float2* p = a.lse_part + (size_t)seg * a.n_slot * a.GW + c0 + e.lane;
-      for (int s0 = first_slot; s0 < n_used; s0 += step * kLseBatch) {
-        float2 pe[NH][kLseBatch];
-#pragma unroll
-        for (int i = 0; i < kLseBatch; ++i)
-#pragma unroll
-          for (int half = 0; half < NH; ++half)
-            pe[half][i] = (s0 + step * i < n_used && e.lane + 32 * half < NC) ? __ldcg(p + (size_t)(s0 + step * i) * a.GW + 32 * half)
-                                                                              : make_float2(-INFINITY, 0.f);
-#pragma unroll
-        for (int half = 0; half < NH; ++half) {
-          float m2 = mx[half];
-#pragma unroll
-          for (int i = 0; i < kLseBatch; ++i) m2 = fmaxf(m2, pe[half][i].x);
-          if (m2 == -INFINITY) continue;
-          if (s0 > first_slot) sum[half] *= exp2f(mx[half] - m2);
-#pragma unroll
-          for (int i = 0; i < kLseBatch; ++i)
-            if (pe[half][i].x != -INFINITY) sum[half] += pe[half][i].y * exp2f(pe[half][i].x - m2);
-          mx[half] = m2;
-        }
-      }
-      if (split) {
-        float2* ex = reinterpret_cast<float2*>(e.xch_s + kXchBytes) + e.wg * 4 * kEpiCols;     // [4 groups][4 warps][64 columns]
-        const uint32_t bar_put = e.bar_norm + 16 * e.wg, bar_got = bar_put + 8;
-        if (!mbar_wait(bar_got, (exchanges + 1) & 1, a.polls, a.poll_ns)) return false;        // passes for the first
-#pragma unroll
-        for (int half = 0; half < NH; ++half) ex[e.quarter * kEpiCols + e.lane + 32 * half] = make_float2(mx[half], sum[half]);
-        __syncwarp();
-        if (e.lane == 0) mbar_arrive(bar_put);
-        if (!mbar_wait(bar_put, exchanges & 1, a.polls, a.poll_ns)) return false;
-#pragma unroll
-        for (int half = 0; half < NH; ++half) {
-          float2 pe[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) pe[i] = ex[i * kEpiCols + e.lane + 32 * half];
-          mx[half] = fmaxf(fmaxf(pe[0].x, pe[1].x), fmaxf(pe[2].x, pe[3].x));
-          sum[half] = 0.f;
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (pe[i].x != -INFINITY) sum[half] += pe[i].y * exp2f(pe[i].x - mx[half]);
-        }
-        __syncwarp();
-        if (e.lane == 0) mbar_arrive(bar_got);
-        ++exchanges;
-      }
-#pragma unroll
-      for (int half = 0; half < NH; ++half) {
-        const int j = e.lane + 32 * half;
-        if (j < NC) {
-          const float lse = mx[half] + log2f(sum[half]);
-          if (tib == 0 && e.quarter == 0) a.lse2[(size_t)seg * a.lse2_stride + a.lse2_off + c0 + j] = lse;
-          lw[j] = -lse;
-        }
-      }
-      __syncwarp();
+      if (!score_normalisers<NC>(a, e, c0, lw, seg, tib, exchanges)) return false;
     }
     float* out = a.s_exact + (size_t)seg * a.S;
     int key = tib * kTileKeys + e.row;

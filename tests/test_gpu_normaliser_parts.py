@@ -1,5 +1,5 @@
 """Segments whose log-sum-exp partials are few enough for every warp of the score pass to fetch them all, and more, so that the
-four warps of a group share the fetching (above eight), for every width of a group's query columns: the scores are those
+four warps of a group share the fetching (above five), for every width of a group's query columns: the scores are those
 of a softmax in fp64. Blocks of one head follow one another, so that a CTA goes from segment to segment."""
 import pytest
 

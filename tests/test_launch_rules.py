@@ -16,6 +16,8 @@ extern "C" int decode_splits(int sms, long long heads, long long len) { return l
 extern "C" int decode_cluster(int sms, long long heads, int group, long long len, const int* room) {
   return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len), room);
 }
+extern "C" int lse_batch() { return lkv::kLseBatch; }
+extern "C" int lse_split(int partials) { return lkv::lse_split(partials); }
 extern "C" int proj_slices(int sms, int grid, long long tiles, int rows, int lse, long long qsig, int abreast, int* begin) {
   const lkv::ProjSlices s = lkv::proj_slices(sms, grid, tiles, rows, lse, qsig, abreast);
   for (int c = 0; s.w_early > 0 && c < grid; ++c) {       // as the kernel: begin and end of every CTA's slice
@@ -72,6 +74,12 @@ def test_clusters_the_device_does_not_hold_are_not_launched(rules, room):
                 assert n == usual or heads > room[usual]       # what fits is launched as ever
                 fewer += n != usual
     assert fewer > 0
+
+
+@pytest.mark.parametrize("partials", range(1, 21))
+def test_normaliser_partials_are_fetched_in_one_round_trip(rules, partials):
+    a_warps = -(-partials // 4) if rules.lse_split(partials) else partials
+    assert a_warps <= rules.lse_batch()
 
 
 def slices(rules, seg_tiles, chunks, rows, qsig, abreast):
