@@ -422,8 +422,6 @@ laser_kv_status_t launch_select(const SelectArgs& a, int n_seg, int num_sms, boo
   return LASER_KV_OK;
 }
 
-// CTAs of an append per SM up to which it starts beside the selection (four are resident at a time).
-constexpr int kAppendBesideCtas = 16;
 int append_ctas(int B) { return (B + kAppendRowsPerCta - 1) / kAppendRowsPerCta; }
 
 laser_kv_status_t launch_append(const AppendArgs& a, int n_seg, cudaStream_t st, bool own_status = false, bool beside = false) {
@@ -844,16 +842,14 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     if (s != LASER_KV_OK) { h->last_error = g_last_error; return s; }
   }
   mark();
-  // 6. gather + append; a grid of a few waves starts beside the selection, which hides its launch (eight segments of
-  //    8192 keys, 488 CTAs: a call 62.9 -> 61.2 us; 64 of 4096, 1856 CTAs: 100.6 -> 99.3). A larger one does not: 7808
-  //    CTAs took 469 instead of 447 us with the layer's other kernels, four sequences of 128k tokens 654 instead of 628.
+  // 6. gather + append, beside the selection where that gains
   {
     const size_t layer_off = (size_t)layer * c.batch * c.n_kv_heads * (size_t)d.cap;
     AppendArgs aa{K0, V0, kv_strides[0], kv_strides[1], kv_strides[2], c.n_kv_heads, nb, S, B, idx,
                   h->cacheK + layer_off * kHeadDim, h->cacheV + layer_off * kHeadDim, h->cachePos + layer_off,
                   d.cap * kHeadDim, d.cap, entries_done, (int)first_token - g.shift, S_len, ctrl};
-    const bool few = (long long)append_ctas(B) * nseg <= (long long)kAppendBesideCtas * h->num_sms && nseg <= h->num_sms;
-    const laser_kv_status_t s = launch_append(aa, nseg, st, false, few && !h->profiling);
+    const bool beside = !h->profiling && append_beside(h->num_sms, nseg, (long long)append_ctas(B) * nseg);
+    const laser_kv_status_t s = launch_append(aa, nseg, st, false, beside);
     if (s != LASER_KV_OK) { h->last_error = g_last_error; return s; }
   }
   mark();

@@ -62,6 +62,17 @@ inline int decode_cluster(int num_sms, long long heads, int group, long long len
   return sixteen && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
 }
 
+// Whether the append of a select call (`ctas` CTAs, four of which an SM holds) is launched beside the selection, which hides its
+// launch: its CTAs then start on the SMs that the selection's leave free. Up to half of the SMs in use by the selection,
+// sixteen CTAs per SM: 24 segments of 2048 keys 42.7 -> 42.3 us a call, 16 of 8192 66.6 -> 65.6, 64 of 4096 (12 per SM) 94.7 ->
+// 95.5 with 10-bit tables and 79.5 either way with 8-bit ones. With more segments the early CTAs crowd onto few SMs: up to eight
+// per SM gain or lose 1 % (128 segments of 1024 keys 53.7 -> 53.3), more lose (80 of 4096, 15 per SM, 113.5 -> 115.5; 128,
+// 11 per SM, 130.0 -> 133.3; 7808 CTAs 447 -> 469, four sequences of 128k tokens 628 -> 654). More segments than SMs: the selection itself
+// starts in waves, and the append is released with the last of them, when there is nothing left to hide.
+inline bool append_beside(int num_sms, int nseg, long long ctas) {
+  return nseg <= num_sms && ctas <= (2 * nseg <= num_sms ? 16ll : 8ll) * num_sms;
+}
+
 // Score pass: log-sum-exp partials of a column that a warp fetches at a time. A segment with more is shared by a group's four warps.
 constexpr int kLseBatch = 5;
 LKV_HOST_DEVICE inline bool lse_split(int partials) { return partials > kLseBatch; }

@@ -16,6 +16,7 @@ extern "C" int decode_splits(int sms, long long heads, long long len) { return l
 extern "C" int decode_cluster(int sms, long long heads, int group, long long len, const int* room) {
   return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len), room);
 }
+extern "C" int append_beside(int sms, int nseg, long long ctas) { return lkv::append_beside(sms, nseg, ctas); }
 extern "C" int lse_batch() { return lkv::kLseBatch; }
 extern "C" int lse_split(int partials) { return lkv::lse_split(partials); }
 extern "C" int proj_slices(int sms, int grid, long long tiles, int rows, int lse, long long qsig, int abreast, int* begin) {
@@ -80,6 +81,16 @@ def test_clusters_the_device_does_not_hold_are_not_launched(rules, room):
 def test_normaliser_partials_are_fetched_in_one_round_trip(rules, partials):
     a_warps = -(-partials // 4) if rules.lse_split(partials) else partials
     assert a_warps <= rules.lse_batch()
+
+
+def test_large_appends_of_many_segments_do_not_start_beside_the_selection(rules):
+    for nseg, rows, beside in ((8, 3855, 1), (64, 1736, 1), (80, 864, 1), (128, 432, 1), (80, 1736, 0), (128, 816, 0), (149, 64, 0),
+                               (128, 3855, 0)):
+        assert rules.append_beside(SMS, nseg, C.c_longlong(-(-rows // 64) * nseg)) == beside
+    # launched early or not, one rule for every number of segments: fewer CTAs never start later
+    for nseg in range(1, 200):
+        early = [rules.append_beside(SMS, nseg, C.c_longlong(ctas)) for ctas in range(1, 3000, 37)]
+        assert early == sorted(early, reverse=True)
 
 
 def slices(rules, seg_tiles, chunks, rows, qsig, abreast):
