@@ -82,27 +82,31 @@ LKV_HOST_DEVICE inline bool lse_split(int partials) { return partials > kLseBatc
 // the selection waited for them. They get fewer tiles, about 5 us less of them (eight of 160 columns), but not less than 55 %:
 // sixteen calls of one block of 8192 tokens 978 -> 953 us (at least 50 %: 959, 60 %: 961, 70 %: 969), 64k in one call
 // 203 -> 198, 32k 101.8 -> 98.8.
-// Where the keys outgrow the L2 cache (above 64 MB), CTAs with the same keys and different chunks must stay together, or the
-// keys come from memory again for each chunk: unequal slices one behind the other took a 128k layer from 399 to 432 us in a
-// burst, slices abreast leave it as it was (four sequences of 128k tokens 622 -> 614 us, 64k 179 -> 176). With keys in the
-// cache the slices one behind the other are the better ones by 1 %.
-constexpr long long kProjAbreastBytes = 64ll << 20;
+// With several chunks of hyperplanes the keys are read once for each, and the slices of the chunks lie abreast: CTAs with the same keys
+// and different chunks stay together. One behind the other, unequal slices took a 128k layer from 399 to 432 us in a burst; abreast
+// they leave it as it was (four sequences of 128k tokens 622 -> 614 us, 64k 179 -> 176). Keys that stay in the L2 cache lose less:
+// 64 MiB 114.1 one behind the other, 113.1 abreast (four chunks), 48 MiB 79.9 / 79.0 (two), 32 MiB 63.7 / 63.2. 16 MiB in segments of 1024
+// keys are better one behind the other, 40.5 / 40.8 and 47.7 / 48.0, hence the line between. Chunks that do not divide the grid
+// cannot lie abreast: up to 64 MiB their slices are unequal one behind the other, above they are equal.
+constexpr long long kProjAbreastBytes = 24ll << 20, kProjUnequalBytes = 64ll << 20;
 struct ProjSlices {
   int n_late, w_late, w_early;   // the last n_late CTAs' slices are to the others' as w_late to w_early; all 0: equal slices
   int abreast;                   // > 1: the sequence is cut into that many equal parts, CTAs c, c + 1, ... at the same place of each
 };
 
-// `grid` CTAs over n_tiles tiles of stat_rows columns, behind a log-sum-exp pass of lse_ctas CTAs that started beside qsig_ctas of the
+// `grid` CTAs over the tiles of `chunks` passes over keys of seg_tiles tiles, stat_rows columns each, behind a log-sum-exp pass of lse_ctas CTAs that started beside qsig_ctas of the
 // query-signature kernel. Late are only the log-sum-exp CTAs that found no SM free: with few tiles in all, weights for every SM
 // with a signature CTA gave some CTAs a second tile for nothing (64 tiles of one head 34.1 us a call with equal slices, 34.9 so
 // weighted; 128 tiles of 16 segments 25.3 / 26.5, of 2 heads 28.4 / 29.9).
-inline ProjSlices proj_slices(int num_sms, int grid, long long n_tiles, int stat_rows, int lse_ctas, long long qsig_ctas, int abreast) {
+inline ProjSlices proj_slices(int num_sms, int grid, long long seg_tiles, int chunks, int stat_rows, int lse_ctas, long long qsig_ctas) {
+  const long long key_bytes = seg_tiles * 128 * 256, n_tiles = seg_tiles * chunks;
+  const bool divides = grid % chunks == 0;
   long long late = lse_ctas + qsig_ctas - num_sms;
   if (late > qsig_ctas) late = qsig_ctas;
-  if (late <= 0 || late >= grid || grid % abreast) return ProjSlices{0, 0, 0, 0};
+  if (late <= 0 || late >= grid || (!divides && key_bytes > kProjUnequalBytes)) return ProjSlices{0, 0, 0, 0};
   const long long per = 1000 * n_tiles / grid, less = 1000ll * 8 * 160 / stat_rows;      // thousandths of a tile
   ProjSlices s;
-  s.abreast = abreast;
+  s.abreast = divides && key_bytes > kProjAbreastBytes ? chunks : 1;
   s.n_late = (int)late;
   s.w_early = (int)(per < 1000000 ? per : 1000000);
   const long long w_less = less * s.w_early / per, most = s.w_early * 45ll / 100;

@@ -19,8 +19,10 @@ extern "C" int decode_cluster(int sms, long long heads, int group, long long len
 extern "C" int append_beside(int sms, int nseg, long long ctas) { return lkv::append_beside(sms, nseg, ctas); }
 extern "C" int lse_batch() { return lkv::kLseBatch; }
 extern "C" int lse_split(int partials) { return lkv::lse_split(partials); }
-extern "C" int proj_slices(int sms, int grid, long long tiles, int rows, int lse, long long qsig, int abreast, int* begin) {
-  const lkv::ProjSlices s = lkv::proj_slices(sms, grid, tiles, rows, lse, qsig, abreast);
+extern "C" int proj_slices(int sms, int grid, long long seg_tiles, int chunks, int rows, int lse, long long qsig, int* begin, int* abreast) {
+  const lkv::ProjSlices s = lkv::proj_slices(sms, grid, seg_tiles, chunks, rows, lse, qsig);
+  const long long tiles = seg_tiles * chunks;
+  *abreast = s.abreast;
   for (int c = 0; s.w_early > 0 && c < grid; ++c) {       // as the kernel: begin and end of every CTA's slice
     const int n = grid / s.abreast;
     const long long part = tiles / s.abreast, first = part * (c % s.abreast);
@@ -93,12 +95,12 @@ def test_large_appends_of_many_segments_do_not_start_beside_the_selection(rules)
         assert early == sorted(early, reverse=True)
 
 
-def slices(rules, seg_tiles, chunks, rows, qsig, abreast):
-    """(CTAs that start late, [begin, end) of every CTA's slice or None where they are equal)."""
+def slices(rules, seg_tiles, chunks, rows, qsig):
+    """(CTAs that start late, [begin, end) of every CTA's slice or None where they are equal, chunks abreast)."""
     lse, grid = min(SMS, seg_tiles), min(SMS, seg_tiles * chunks)
-    out = (C.c_int * (2 * grid))()
-    late = rules.proj_slices(SMS, grid, C.c_longlong(seg_tiles * chunks), rows, lse, C.c_longlong(qsig), abreast, out)
-    return late, list(zip(out[::2], out[1::2])) if late else None
+    out, abreast = (C.c_int * (2 * grid))(), C.c_int()
+    late = rules.proj_slices(SMS, grid, C.c_longlong(seg_tiles), chunks, rows, lse, C.c_longlong(qsig), out, C.byref(abreast))
+    return late, list(zip(out[::2], out[1::2])) if late else None, abreast.value
 
 
 @pytest.mark.parametrize("rows", [64, 128, 160, 192])
@@ -107,20 +109,24 @@ def test_slices_of_the_projection_pass_are_the_tiles_in_turn(rules, rows):
     for seg_tiles in list(range(1, 300, 7)) + [1024, 8192, 65536, 300000]:
         for chunks in (1, 2, 3, 4, 5, 8):
             for qsig in (1, 4, 16, 64, 147, 148, 500):
-                for abreast in {1, chunks}:
-                    late, cut = slices(rules, seg_tiles, chunks, rows, qsig, abreast)
-                    if cut is None:
-                        continue
-                    weighted += 1
-                    assert 0 < late <= qsig and all(b <= e for b, e in cut)
-                    ends = sorted(x for x in cut if x[0] < x[1])
-                    assert ends[0][0] == 0 and ends[-1][1] == seg_tiles * chunks
-                    assert all(a[1] == b[0] for a, b in zip(ends, ends[1:]))
+                late, cut, abreast = slices(rules, seg_tiles, chunks, rows, qsig)
+                if cut is None:
+                    continue
+                weighted += 1
+                assert 0 < late <= qsig and all(b <= e for b, e in cut)
+                ends = sorted(x for x in cut if x[0] < x[1])
+                assert ends[0][0] == 0 and ends[-1][1] == seg_tiles * chunks
+                assert all(a[1] == b[0] for a, b in zip(ends, ends[1:]))
+                if seg_tiles * 128 * 256 > 24 << 20:           # neighbours read the same keys
+                    assert abreast == (chunks if SMS % chunks == 0 else 1)
+                    for i in range(0, len(cut) - abreast, abreast):
+                        places = [cut[i + k][0] - k * seg_tiles * chunks // abreast for k in range(abreast)]
+                        assert max(places) == min(places)
     assert weighted > 100
 
 
 @pytest.mark.parametrize("seg_tiles,chunks,qsig", [(48, 1, 4), (64, 1, 16), (64, 2, 4), (84, 4, 64), (96, 1, 16), (128, 1, 16), (132, 1, 16)])
 def test_slices_are_equal_where_no_cta_starts_late(rules, seg_tiles, chunks, qsig):
     # every log-sum-exp CTA finds an SM without a signature CTA: a slice of two tiles beside one of none would take a tile longer
-    assert slices(rules, seg_tiles, chunks, 160, qsig, 1) == (0, None)
-    assert slices(rules, SMS - qsig + 1, chunks, 160, qsig, 1)[0] == 1
+    assert slices(rules, seg_tiles, chunks, 160, qsig)[:2] == (0, None)
+    assert slices(rules, SMS - qsig + 1, chunks, 160, qsig)[0] == 1
