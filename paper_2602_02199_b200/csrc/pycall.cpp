@@ -1,7 +1,8 @@
 // Native call path of the Python binding for the entry points that run once per layer, block or token: argument
 // conversion and the call itself, without ctypes. A call takes tensor addresses, sizes and torch's stride tuples and returns
 // the status. One decoded token through 32 layers whose kernels take 5 us each was bound by the host at 8.2 us a layer.
-// Integers are taken modulo the width of the parameter, as ctypes takes them; the interpreter lock is released during the call.
+// What ctypes takes is taken: for a number whatever says that it is an integer (__index__: numpy's integers, tensors of one element),
+// modulo the width of the parameter, for a pointer an int; the interpreter lock is released during the call.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <dlfcn.h>
@@ -24,16 +25,21 @@ struct Args {
   PyObject* const* p;
   bool ok = true;
   long long integer(PyObject* o) {
-    if (!PyLong_Check(o)) {
-      if (ok) PyErr_Format(PyExc_TypeError, "int expected instead of %s", Py_TYPE(o)->tp_name);
-      ok = false;
-      return 0;
-    }
-    return (long long)PyLong_AsUnsignedLongLongMask(o);
+    if (!ok) return 0;
+    const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
+    if (v == (unsigned long long)-1 && PyErr_Occurred()) ok = false;
+    return (long long)v;
   }
   long long i64() { return integer(*p++); }
   int32_t i32() { return (int32_t)i64(); }
-  void* ptr() { return reinterpret_cast<void*>(i64()); }
+  void* ptr() {
+    PyObject* o = *p++;
+    if (ok && !PyLong_Check(o)) {
+      PyErr_Format(PyExc_TypeError, "address expected as int instead of %s", Py_TYPE(o)->tp_name);
+      ok = false;
+    }
+    return reinterpret_cast<void*>(integer(o));
+  }
   float f32() {
     PyObject* o = *p++;
     if (!ok) return 0.f;

@@ -2,6 +2,7 @@
 not a call is refused."""
 import numpy as np
 import pytest
+import torch
 
 from paper_2602_02199_b200 import binding as Bn
 
@@ -43,13 +44,31 @@ def test_every_argument_reaches_its_parameter(native):
     assert native.two_stage_topk(16, 16, (1 << 32) + 1, 16385, 1, 1, 1, 16, 0) == Bn.ERR_UNSUPPORTED
 
 
+class _Seven:
+    def __index__(self):
+        return 7
+
+
+@pytest.mark.parametrize("seven", [7, np.int64(7), np.uint8(7), torch.tensor(7), _Seven()], ids=lambda x: type(x).__name__)
+def test_numbers_are_whatever_ctypes_takes_for_an_integer(native, seven):
+    big = 1 << 40
+    assert native.gather_append(16, 16, 8, 8, 5, 16, 1, seven, 16, 16, 8, np.int64(big + 6), 16, 8, np.int64(big), 0, 16, 0) == Bn.ERR_CAPACITY
+    assert f"[{big}, {big + 7})" in _message() and f"{big + 6} entries" in _message()
+    lib = Bn.load()                                      # the same arguments by way of ctypes
+    assert lib.laser_kv_gather_append(16, 16, 8, 8, 5, 16, 1, seven, 16, 16, 8, np.int64(big + 6), 16, 8, np.int64(big), 0, 16, 0) == Bn.ERR_CAPACITY
+    st = (128, seven, np.int32(128), 1)
+    assert native.window_scores(16, 16, st, st, 1, 4, 1, 64, 16, 2, 0.5, 256, 100, 16, 0) == Bn.ERR_CAPACITY
+
+
 def test_what_is_not_a_call_raises(native):
     with pytest.raises(TypeError):
         native.two_stage_topk(0, 0)
     with pytest.raises(TypeError):
         native.two_stage_topk(0, 0, 1.5, 8, 1, 1, 1, 0, 0)
     with pytest.raises(TypeError):
-        native.two_stage_topk(0, 0, np.int64(1), 8, 1, 1, 1, 0, 0)
+        native.two_stage_topk(0, 0, np.float64(1), 8, 1, 1, 1, 0, 0)
+    with pytest.raises(TypeError):
+        native.two_stage_topk(np.int64(0), 0, 1, 8, 1, 1, 1, 0, 0)             # an address
     with pytest.raises(ValueError):
         native.decode_attention(0, 0, 16, (128,), 0.0, 16, 16, 64, 0)
     with pytest.raises(ValueError):
