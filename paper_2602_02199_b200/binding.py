@@ -156,6 +156,7 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     lib.laser_kv_decode_attention_scratch_bytes.argtypes = [vp]
     lib.laser_kv_decode_attention.restype = i32
     lib.laser_kv_decode_attention.argtypes = [vp, i32, vp, p(i64), C.c_float, vp, vp, sz, vp]
+    importlib.invalidate_caches()      # it may have been built a moment ago
     native = importlib.import_module("._pycall", __package__)
     native.setup(_build.LIB)
     _pycall, _lib = native, lib

@@ -27,6 +27,21 @@ def _older(target: str, deps: list) -> bool:
     return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
 
 
+def _link(cmd: list, target: str, what: str) -> str:
+    """Runs a compiler that writes `target`, by way of a file of this process's own: another process that loads or builds the same
+    file sees all of it or none."""
+    part = f"{target}.{os.getpid()}.so"
+    try:
+        res = subprocess.run(cmd + ["-o", part], capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError(what + " failed:\n" + res.stdout + res.stderr)
+        os.replace(part, target)
+    finally:
+        if os.path.exists(part):
+            os.remove(part)
+    return res.stderr
+
+
 def needs_build() -> bool:
     return _older(LIB, [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [API])
 
@@ -38,10 +53,8 @@ def _build_pycall(force: bool) -> None:
     cxx = os.environ.get("CXX") or shutil.which("g++") or shutil.which("c++")
     if not cxx:
         raise RuntimeError("no C++ compiler found; one is required to build the binding's native call path")
-    res = subprocess.run([cxx, "-shared", "-fPIC", "-O2", "-std=c++17", "-I", sysconfig.get_paths()["include"], "-o", PYCALL, src],
-                         capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("building the binding's native call path failed:\n" + res.stdout + res.stderr)
+    _link([cxx, "-shared", "-fPIC", "-O2", "-std=c++17", "-I", sysconfig.get_paths()["include"], src], PYCALL,
+          "building the binding's native call path")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -49,15 +62,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
     cmd = [_nvcc(), "-shared", "-Xcompiler", "-fPIC", "-gencode", "arch=compute_100a,code=sm_100a",
-           "-lineinfo", "-O3", "-std=c++17", "-o", LIB] + [os.path.join(CSRC, s) for s in SOURCES]
+           "-lineinfo", "-O3", "-std=c++17"] + [os.path.join(CSRC, s) for s in SOURCES]
     if verbose:
         cmd.insert(1, "-Xptxas")
         cmd.insert(2, "-v")
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+    log = _link(cmd, LIB, "nvcc")
     if verbose:
-        print(res.stderr)
+        print(log)
     return LIB
 
 
