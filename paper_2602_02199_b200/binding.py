@@ -6,6 +6,7 @@ from __future__ import annotations
 import ctypes as C
 import importlib
 import os
+import warnings
 from dataclasses import dataclass
 
 from . import build as _build
@@ -66,7 +67,35 @@ class LaserKVError(RuntimeError):
 
 
 _lib = None
-_pycall = None      # the native call path, loaded with the library
+_pycall = None      # the native call path, or the same calls by way of ctypes, chosen when the library is loaded
+
+
+class _CtypesCalls:
+    """The calls of the native call path by way of ctypes, which takes 2 to 3 us more of host time for each."""
+
+    def __init__(self, lib):
+        self._lib = lib
+
+    def __getattr__(self, name):
+        function = getattr(self._lib, "laser_kv_" + name)
+
+        def call(*args):
+            return function(*[(C.c_int64 * max(3, len(a)))(*a) if isinstance(a, tuple) else a for a in args])    # stride tuples
+        setattr(self, name, call)
+        return call
+
+
+def _native_calls(lib, build_if_missing: bool):
+    try:
+        if build_if_missing:
+            _build.build_pycall()
+        importlib.invalidate_caches()      # it may have been built a moment ago
+        native = importlib.import_module("._pycall", __package__)
+        native.setup(_build.LIB)
+        return native
+    except (RuntimeError, ImportError, OSError) as e:
+        warnings.warn(f"calls go by way of ctypes, which costs 2 to 3 us of host time each: {e}")
+        return _CtypesCalls(lib)
 
 
 def lib_path() -> str:
@@ -79,7 +108,7 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     if _lib is not None:
         return _lib
     if build_if_missing:
-        _build.build()      # a no-op when the library is newer than its sources; a failed rebuild raises
+        _build.build_lib()      # a no-op when the library is newer than its sources; a failed rebuild raises
     if not os.path.exists(_build.LIB):
         raise RuntimeError(f"{_build.LIB} is missing: build it with python -m paper_2602_02199_b200.build")
     lib = C.CDLL(_build.LIB)
@@ -156,10 +185,7 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     lib.laser_kv_decode_attention_scratch_bytes.argtypes = [vp]
     lib.laser_kv_decode_attention.restype = i32
     lib.laser_kv_decode_attention.argtypes = [vp, i32, vp, p(i64), C.c_float, vp, vp, sz, vp]
-    importlib.invalidate_caches()      # it may have been built a moment ago
-    native = importlib.import_module("._pycall", __package__)
-    native.setup(_build.LIB)
-    _pycall, _lib = native, lib
+    _pycall, _lib = _native_calls(lib, build_if_missing), lib
     return lib
 
 

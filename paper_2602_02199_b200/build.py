@@ -3,6 +3,7 @@ native call path."""
 from __future__ import annotations
 
 import os
+import shlex
 import shutil
 import subprocess
 import sysconfig
@@ -46,19 +47,23 @@ def needs_build() -> bool:
     return _older(LIB, [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [API])
 
 
-def _build_pycall(force: bool) -> None:
+def build_pycall(force: bool = False) -> None:
     src = os.path.join(CSRC, "pycall.cpp")
     if not force and not _older(PYCALL, [src, API]):
         return
-    cxx = os.environ.get("CXX") or shutil.which("g++") or shutil.which("c++")
-    if not cxx:
+    cxx = shlex.split(os.environ.get("CXX") or "") or [c for c in ("g++", "c++") if shutil.which(c)][:1]
+    if not cxx or not shutil.which(cxx[0]):
         raise RuntimeError("no C++ compiler found; one is required to build the binding's native call path")
-    _link([cxx, "-shared", "-fPIC", "-O2", "-std=c++17", "-I", sysconfig.get_paths()["include"], src], PYCALL,
+    _link(cxx + ["-shared", "-fPIC", "-O2", "-std=c++17", "-I", sysconfig.get_paths()["include"], src], PYCALL,
           "building the binding's native call path")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    _build_pycall(force)
+    build_pycall(force)
+    return build_lib(force, verbose)
+
+
+def build_lib(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
     cmd = [_nvcc(), "-shared", "-Xcompiler", "-fPIC", "-gencode", "arch=compute_100a,code=sm_100a",
