@@ -1,5 +1,5 @@
-"""Decode attention at the cache lengths where the number of splits changes its rule (eight tiles, 24
-tiles, three tiles per split), against fp64. The numerators keep 24 bits: what is left is the rounding of the
+"""Decode attention over one to 112 tiles, which merge in clusters of up to eight and of sixteen splits, against fp64
+(test_gpu_decode_memory.py has the shapes whose splits merge by way of memory). The numerators keep 24 bits: what is left is the rounding of the
 fp32 sums, 1.0e-7 (one tile) to 3.1e-7 of the result's norm over these lengths and six seeds each. Numerators of
 two bf16 terms, 2^-17 off at most, would leave 1.3e-6 to 2.4e-6: the bound of 8e-7 tells the two apart."""
 import pytest

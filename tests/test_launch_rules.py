@@ -6,6 +6,8 @@ import subprocess
 
 import pytest
 
+import test_gpu_decode_memory as memory
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_02199_b200", "csrc")
 SMS = 148
 # clusters of 0 to 16 decode CTAs that such a device holds at once (9 to 15 are not used)
@@ -64,6 +66,12 @@ def test_few_heads_give_no_cta_more_than_six_tiles_of_a_short_cache(rules, heads
     for group in range(1, 9):
         for tiles in range(1, 65):
             assert -(-tiles // cluster(rules, heads, group, 64 * tiles)) <= 6
+
+
+def test_the_shapes_of_the_memory_route_take_it(rules):
+    for shape in memory.SHAPES:
+        batch, heads, group = shape[:3]
+        assert cluster(rules, batch * heads, group, memory.entries(shape)) == 0
 
 
 @pytest.mark.parametrize("room", [[0] * 17, [0, 0] + [1] * 7 + [0] * 8, ROOM[:9] + [0] * 8, [n // 4 for n in ROOM]])
