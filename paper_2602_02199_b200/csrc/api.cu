@@ -77,7 +77,7 @@ struct laser_kv_ctx {
   CUtensorMap mapPq;   // hyperplanes, box = the eight tables of one query-signature CTA
   EncodeTiledFn encode = nullptr;
   int num_sms = 1;
-  int cluster_room[kDecMaxCluster + 1] = {0};   // decode: clusters of each size that the device holds at once
+  int cluster_room[kDecMaxCluster + 1] = {0};   // decode: 1 + the clusters of each size that the device holds at once; 0: not asked yet
   std::vector<long long> blocks_done;   // per layer: blocks processed
   std::vector<long long> entries_done;  // per layer: cache entries final per (sequence, KV head)
   std::vector<long long> tokens_done;   // per layer: tokens of the blocks processed
@@ -542,8 +542,6 @@ laser_kv_status_t laser_kv_init(const laser_kv_config_t* cfg, const void* hyperp
   h->ws = static_cast<uint8_t*>(workspace);
   h->encode = reinterpret_cast<EncodeTiledFn>(fn);
   h->num_sms = prop.multiProcessorCount;
-  for (int n = 2; n <= 8; ++n) h->cluster_room[n] = decode_cluster_room<8>(n);
-  h->cluster_room[16] = decode_cluster_room<16>(16);
   const size_t per = (size_t)cfg->n_layers * cfg->batch * cfg->n_kv_heads * (size_t)d.cap;
   uint8_t* cm = static_cast<uint8_t*>(cache_mem);
   h->cacheK = reinterpret_cast<uint16_t*>(cm);
@@ -1217,7 +1215,11 @@ laser_kv_status_t laser_kv_decode_attention(laser_kv_handle_t h, int32_t layer, 
   a.counters = reinterpret_cast<int*>(h->ws + h->carve.dec_count);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e;
-  const int n_cluster = decode_cluster(h->num_sms, heads, G, len, n_split, h->cluster_room);
+  const int n_cluster = decode_cluster(h->num_sms, heads, G, len, n_split, [h](int n) {
+    int& room = h->cluster_room[n];
+    if (!room) room = 1 + (n <= 8 ? decode_cluster_room<8>(n) : decode_cluster_room<16>(n));
+    return room - 1;
+  });
   auto run = [&](auto kernel, cudaError_t limits, int n, int cluster) {
     if (limits != cudaSuccess) return limits;
     a.n_split = n;

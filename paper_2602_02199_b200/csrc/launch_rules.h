@@ -45,21 +45,21 @@ inline int decode_splits(int num_sms, long long heads, long long len) {
 // percent; for three to five the clusters it takes are up to 7 % slower at single lengths (5 heads of three, 320 tiles 14.9 /
 // 16.0; 4 of four, 100 7.3 / 7.7) and up to 13 % faster at others (6 of four, 80 8.1 / 7.0), and 2.1e-7 instead of 2.7e-7
 // to 4e-7 from fp64.
-// `room`: how many clusters of each size (up to kDecMaxCluster) the device holds at once. Only sizes of which it holds
-// all the call's are used; a device, or a part of one, that holds none of a size would refuse the launch. The B200's
-// 148 SMs hold 33 of eight, 14 of sixteen.
-inline int decode_cluster(int num_sms, long long heads, int group, long long len, int n_split, const int* room) {
+// `room(n)`: how many clusters of n (up to kDecMaxCluster) the device holds at once; asked only of a size about to be used. Only
+// sizes of which it holds all the call's are used; a device, or a part of one, that holds none of a size would refuse the
+// launch. The B200's 148 SMs hold 33 of eight, 14 of sixteen.
+template <typename Room>
+inline int decode_cluster(int num_sms, long long heads, int group, long long len, int n_split, Room&& room) {
   const long long tiles = (len + kDecTile - 1) / kDecTile;
-  const bool sixteen = 16 * heads <= num_sms && heads <= room[16];
   if (tiles <= 64) {
-    if (tiles > 48 && heads <= 6 && sixteen) return 16;
+    if (tiles > 48 && heads <= 6 && 16 * heads <= num_sms && heads <= room(16)) return 16;
     long long n = (long long)num_sms * kDecCtasPerSm / heads;
     if (n > 8) n = 8;
     if (n > tiles) n = tiles;
     if (n <= 1) return 1;
-    return n * heads <= 256 && heads <= room[n] ? (int)n : 0;
+    return n * heads <= 256 && heads <= room((int)n) ? (int)n : 0;
   }
-  return sixteen && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) ? 16 : 0;
+  return 16 * heads <= num_sms && 3 * ((long long)group * n_split - 60) > tiles * (heads < 5 ? 6 - heads : 1) && heads <= room(16) ? 16 : 0;
 }
 
 // Whether the append of a select call (`ctas` CTAs, four of which an SM holds) is launched beside the selection, which hides its

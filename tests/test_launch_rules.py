@@ -16,7 +16,7 @@ SHIM = """
 #include "launch_rules.h"
 extern "C" int decode_splits(int sms, long long heads, long long len) { return lkv::decode_splits(sms, heads, len); }
 extern "C" int decode_cluster(int sms, long long heads, int group, long long len, const int* room) {
-  return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len), room);
+  return lkv::decode_cluster(sms, heads, group, len, lkv::decode_splits(sms, heads, len), [=](int n) { return room[n]; });
 }
 extern "C" int append_beside(int sms, int nseg, long long ctas) { return lkv::append_beside(sms, nseg, ctas); }
 extern "C" int lse_batch() { return lkv::kLseBatch; }
