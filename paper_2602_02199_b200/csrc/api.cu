@@ -826,7 +826,7 @@ laser_kv_status_t run_select(laser_kv_ctx* h, int layer, const void* K_blk, cons
     const int grid = stream_grid(a3.n_tiles, h->num_sms);
     if (need_exact && !h->profiling)
       a3.slices = proj_slices(h->num_sms, grid, seg_tiles, d.n_chunks, a3.stat_rows, base_ctas,
-                              (long long)d.Lp / kQsigTables * c.n_kv_heads * c.batch);
+                              (long long)d.Lp / kQsigTables * c.n_kv_heads * c.batch, d.n_qparts);
     a3.fix_list = fix_list_items(d.fix_cap, (size_t)d.nseg_max, grid);
     LKV_CUDA(launch_proj(d.Kp, d.TC, mapK, h->mapP, a3, grid, smem, st),
              "projection pass");

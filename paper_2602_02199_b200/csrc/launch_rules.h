@@ -41,10 +41,11 @@ inline int decode_splits(int num_sms, long long heads, long long len) {
 // Longer caches of few heads with many queries: the general path's merge costs as much as its partials are large, a cluster
 // of sixteen reads the cache with fewer CTAs (one head of eight, 512 tiles 28.4 / 18.5; 4 heads of seven, 160 15.5 / 10.7, 512
 // 24.4 / 21.2, 1024 35.1 / 36.2; 8 heads of four, 80 8.3 / 8.5, 255 16.8 / 16.7, 512 27.0 / 27.4; 4 heads of two, 80 6.4 / 6.5).
-// The inequality is where the two cross for 1 to 9 heads and twelve lengths of 70 to 1024 tiles: at six queries and more to a
-// percent; for three to five the clusters it takes are up to 7 % slower at single lengths (5 heads of three, 320 tiles 14.9 /
-// 16.0; 4 of four, 100 7.3 / 7.7) and up to 13 % faster at others (6 of four, 80 8.1 / 7.0), and 2.1e-7 instead of 2.7e-7
-// to 4e-7 from fp64.
+// The inequality is where the two cross for 1 to 9 heads and twelve lengths of 70 to 1024 tiles over four layers' caches. Where the
+// caches of more layers come from memory in turn, clusters gain more: 16 layers, 8 heads of four, 66 tiles 9.0 / 8.7, 98 10.4 / 10.0, 160
+// 13.2 / 12.4; 8 of five, 130 13.2 / 11.6; 9 of four, 80 9.9 / 9.2; 5 of three, 160 the same. Two layers, which the L2 cache holds,
+// are up to 17 % slower of three to five queries (8 heads of four, 98 tiles 8.3 / 9.3): not what a model's decoding looks like. The
+// results are 2.1e-7 instead of 2.7e-7 to 4e-7 from fp64 (normal keys, values and queries).
 // `room(n)`: how many clusters of n (up to kDecMaxCluster) the device holds at once; asked only of a size about to be used. Only
 // sizes of which it holds all the call's are used; a device, or a part of one, that holds none of a size would refuse the
 // launch. The B200's 148 SMs hold 33 of eight, 14 of sixteen.
@@ -97,13 +98,15 @@ struct ProjSlices {
 // `grid` CTAs over the tiles of `chunks` passes over keys of seg_tiles tiles, stat_rows columns each, behind a log-sum-exp pass of lse_ctas CTAs that started beside qsig_ctas of the
 // query-signature kernel. Late are only the log-sum-exp CTAs that found no SM free: with few tiles in all, weights for every SM
 // with a signature CTA gave some CTAs a second tile for nothing (64 tiles of one head 34.1 us a call with equal slices, 34.9 so
-// weighted; 128 tiles of 16 segments 25.3 / 26.5, of 2 heads 28.4 / 29.9).
-inline ProjSlices proj_slices(int num_sms, int grid, long long seg_tiles, int chunks, int stat_rows, int lse_ctas, long long qsig_ctas) {
+// weighted; 128 tiles of 16 segments 25.3 / 26.5, of 2 heads 28.4 / 29.9). A window scored in parts has an ordinary launch between the
+// parts, behind which all CTAs start alike (144 segments of 1016 keys, 320 queries a head, 106.8 / 108.6).
+inline ProjSlices proj_slices(int num_sms, int grid, long long seg_tiles, int chunks, int stat_rows, int lse_ctas, long long qsig_ctas,
+                              int window_parts) {
   const long long key_bytes = seg_tiles * 128 * 256, n_tiles = seg_tiles * chunks;
   const bool divides = grid % chunks == 0;
   long long late = lse_ctas + qsig_ctas - num_sms;
   if (late > qsig_ctas) late = qsig_ctas;
-  if (late <= 0 || late >= grid || (!divides && key_bytes > kProjUnequalBytes)) return ProjSlices{0, 0, 0, 0};
+  if (window_parts > 1 || late <= 0 || late >= grid || (!divides && key_bytes > kProjUnequalBytes)) return ProjSlices{0, 0, 0, 0};
   const long long per = 1000 * n_tiles / grid, less = 1000ll * 8 * 160 / stat_rows;      // thousandths of a tile
   ProjSlices s;
   s.abreast = divides && key_bytes > kProjAbreastBytes ? chunks : 1;

@@ -21,8 +21,8 @@ extern "C" int decode_cluster(int sms, long long heads, int group, long long len
 extern "C" int append_beside(int sms, int nseg, long long ctas) { return lkv::append_beside(sms, nseg, ctas); }
 extern "C" int lse_batch() { return lkv::kLseBatch; }
 extern "C" int lse_split(int partials) { return lkv::lse_split(partials); }
-extern "C" int proj_slices(int sms, int grid, long long seg_tiles, int chunks, int rows, int lse, long long qsig, int* begin, int* abreast) {
-  const lkv::ProjSlices s = lkv::proj_slices(sms, grid, seg_tiles, chunks, rows, lse, qsig);
+extern "C" int proj_slices(int sms, int grid, long long seg_tiles, int chunks, int rows, int lse, long long qsig, int parts, int* begin, int* abreast) {
+  const lkv::ProjSlices s = lkv::proj_slices(sms, grid, seg_tiles, chunks, rows, lse, qsig, parts);
   const long long tiles = seg_tiles * chunks;
   *abreast = s.abreast;
   for (int c = 0; s.w_early > 0 && c < grid; ++c) {       // as the kernel: begin and end of every CTA's slice
@@ -103,11 +103,11 @@ def test_large_appends_of_many_segments_do_not_start_beside_the_selection(rules)
         assert early == sorted(early, reverse=True)
 
 
-def slices(rules, seg_tiles, chunks, rows, qsig):
+def slices(rules, seg_tiles, chunks, rows, qsig, parts=1):
     """(CTAs that start late, [begin, end) of every CTA's slice or None where they are equal, chunks abreast)."""
     lse, grid = min(SMS, seg_tiles), min(SMS, seg_tiles * chunks)
     out, abreast = (C.c_int * (2 * grid))(), C.c_int()
-    late = rules.proj_slices(SMS, grid, C.c_longlong(seg_tiles), chunks, rows, lse, C.c_longlong(qsig), out, C.byref(abreast))
+    late = rules.proj_slices(SMS, grid, C.c_longlong(seg_tiles), chunks, rows, lse, C.c_longlong(qsig), parts, out, C.byref(abreast))
     return late, list(zip(out[::2], out[1::2])) if late else None, abreast.value
 
 
@@ -138,3 +138,5 @@ def test_slices_are_equal_where_no_cta_starts_late(rules, seg_tiles, chunks, qsi
     # every log-sum-exp CTA finds an SM without a signature CTA: a slice of two tiles beside one of none would take a tile longer
     assert slices(rules, seg_tiles, chunks, 160, qsig)[:2] == (0, None)
     assert slices(rules, SMS - qsig + 1, chunks, 160, qsig)[0] == 1
+    # a window scored in parts: an ordinary launch between the parts lets every CTA start alike
+    assert slices(rules, 8192, chunks, 160, qsig)[0] == qsig and slices(rules, 8192, chunks, 160, qsig, parts=2)[0] == 0
