@@ -36,7 +36,7 @@ inline int decode_splits(int num_sms, long long heads, long long len) {
 // up to 256 CTAs in all do (264 of them 10.3 against 10.7, 280 14.3 against 10.8).
 // With few heads eight CTAs of more than six tiles each fall behind splits that have an SM each; a cluster of sixteen does not:
 // 4 heads of one query and 64 tiles 6.3 by way of memory / 7.0 eight / 6.4 sixteen, of four 6.7 / 7.2 / 6.5, 2 heads of two
-// and 50 tiles 6.4 / 6.6 / 6.2, 7 heads of one and 56 6.4 / 6.6 / 6.4, of eight and 64 10.4 / 7.3 / 6.6. From 8 heads on clusters of
+// and 50 tiles 6.4 / 6.6 / 6.2, 6 heads of eight and 64 0.79 / 0.72 of the time by way of memory. From 8 heads on clusters of
 // sixteen share SMs and are slower (8 heads of one, 50 tiles 6.5 / 6.7 / 7.2).
 // Longer caches of few heads with many queries: the general path's merge costs as much as its partials are large, a cluster
 // of sixteen reads the cache with fewer CTAs (one head of eight, 512 tiles 28.4 / 18.5; 4 heads of seven, 160 15.5 / 10.7, 512
@@ -53,7 +53,7 @@ template <typename Room>
 inline int decode_cluster(int num_sms, long long heads, int group, long long len, int n_split, Room&& room) {
   const long long tiles = (len + kDecTile - 1) / kDecTile;
   if (tiles <= 64) {
-    if (tiles > 48 && heads <= 7 && 16 * heads <= num_sms && heads <= room(16)) return 16;
+    if (tiles > 48 && heads <= 6 && 16 * heads <= num_sms && heads <= room(16)) return 16;
     long long n = (long long)num_sms * kDecCtasPerSm / heads;
     if (n > 8) n = 8;
     if (n > tiles) n = tiles;

@@ -60,7 +60,7 @@ def test_decode_splits_are_whole_tiles_and_never_empty(rules):
             assert 1 <= n <= min(tiles, 512) and 0 <= c <= min(tiles, 16)
 
 
-@pytest.mark.parametrize("heads", [1, 2, 3, 4, 5, 6, 7])
+@pytest.mark.parametrize("heads", [1, 2, 3, 4, 5, 6])
 def test_few_heads_give_no_cta_more_than_six_tiles_of_a_short_cache(rules, heads):
     # seven and eight tiles a CTA cost up to 12 % against splits by way of memory that have an SM each
     for group in range(1, 9):
