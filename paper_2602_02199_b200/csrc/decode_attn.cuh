@@ -18,8 +18,8 @@
 //                           numerators relative to the warp's running reference maximum (raised
 //                           only when a score exceeds it by 2^20), O^T += V^T P^T with the
 //                           numerators split into three bf16 terms so that the weights keep all
-//                           24 bits (two terms: 2.0e-6 instead of 3.4e-7 from fp64 over 1636 entries
-//                           when a split had one accumulator; the third costs 0.4 us of 43 over
+//                           24 bits (two terms leave 2.0e-6 from fp64 over 1636 entries, three 2.2e-7
+//                           or less, see below; the third costs 0.4 us of 43 over
 //                           61680, 1.7 of 150 for four such sequences; issuing the MMAs of 2, 4 or 8 row blocks term
 //                           by term, so that they do not wait for one another, changes neither).
 //                           -> partial (max, sum, G x 128 accumulator) per split.
