@@ -39,11 +39,11 @@ UNIT = "tokens/s"
 # summary of the select call, keyed by (workload, kernel). A missing key means: not captured for
 # this workload, or the kernel has changed since the capture.
 NCU_TRAFFIC_BYTES = {
-    ("llama8b_128k", "stream_kernel<proj>"): 281520128 + 3959552,
-    ("llama8b_128k", "stream_kernel<lse>"): 269275648 + 629504,
-    ("llama8b_128k", "stream_kernel<score>"): 270542080 + 3974144,
-    ("llama8b_128k", "append_kernel"): 254752000 + 200093184,
-    ("llama8b_128k", "select_kernel"): 8416768,
+    ("llama8b_128k", "stream_kernel<proj>"): 280621056 + 3529344,
+    ("llama8b_128k", "stream_kernel<lse>"): 269298304 + 273920,
+    ("llama8b_128k", "stream_kernel<score>"): 270209408 + 2606592,
+    ("llama8b_128k", "append_kernel"): 254673792 + 195084416,
+    ("llama8b_128k", "select_kernel"): 8420096 + 3968,
     ("llama8b_128k", "decode_split_kernel"): 252766464 + 512512,
 }
 

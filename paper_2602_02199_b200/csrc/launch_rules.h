@@ -37,7 +37,8 @@ inline int decode_splits(int num_sms, long long heads, long long len) {
 // With few heads eight CTAs of more than six tiles each fall behind splits that have an SM each; a cluster of sixteen does not:
 // 4 heads of one query and 64 tiles 6.3 by way of memory / 7.0 eight / 6.4 sixteen, of four 6.7 / 7.2 / 6.5, 2 heads of two
 // and 50 tiles 6.4 / 6.6 / 6.2, 6 heads of eight and 64 0.79 / 0.72 of the time by way of memory. From 8 heads on clusters of
-// sixteen share SMs and are slower (8 heads of one, 50 tiles 6.5 / 6.7 / 7.2).
+// sixteen share SMs and are slower (8 heads of one, 50 tiles 6.5 / 6.7 / 7.2); with 7, of one over 56 tiles, 6.4 / 6.6 / 6.4
+// over four layers' caches, but 7.7 / 7.5 / 7.7 over 24, which come from memory.
 // Longer caches of few heads with many queries: the general path's merge costs as much as its partials are large, a cluster
 // of sixteen reads the cache with fewer CTAs (one head of eight, 512 tiles 28.4 / 18.5; 4 heads of seven, 160 15.5 / 10.7, 512
 // 24.4 / 21.2, 1024 35.1 / 36.2; 8 heads of four, 80 8.3 / 8.5, 255 16.8 / 16.7, 512 27.0 / 27.4; 4 heads of two, 80 6.4 / 6.5).
